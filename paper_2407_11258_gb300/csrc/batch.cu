@@ -62,7 +62,7 @@ long long estimate_fragment_bytes(int o_, int v_, int N_, bool mixed, int n_refi
   b += 8 * (np_v * np_o + nm_v * nm_o + N * ov);
   b += 8 * 2 * std::min(diis, 8) * L;
   const long long cap = packing_scratch_elems(o_, v_, N_);
-  b += 2 * 8 * cap + 8 * (1LL << 22);
+  b += 2 * 8 * cap + 8 * (1LL << 22) + static_cast<long long>(slice_ws_bytes(8 * static_cast<size_t>(cap)));
   auto consts = [&](long long esz) {
     long long c = np_o * kp(np_v) + nm_o * kp(nm_v) + (2 * ov + oo + vv) * kp(N) + oo * kp(vv) + 2 * ov * kp(ov) +
                   v * kp(oo * v) + ov * kp(vv) + np_v * kp(np_v) + nm_v * kp(nm_v);

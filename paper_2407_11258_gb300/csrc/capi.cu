@@ -266,6 +266,14 @@ int lnocc_debug_gemm(int precision, int M, int N, int K, const double* A, const 
   double* ws = nullptr;
   LN_CUDA(cudaMalloc(&ws, (1u << 22) * sizeof(double)));
   lnocc::split_ws() = lnocc::SplitWs{ws, 1u << 22};
+  void* sl = nullptr;
+  if (!bf) {  // digit planes of an FP64 product
+    const size_t nsl = lnocc::slice_ws_bytes(static_cast<size_t>(std::max(M, N)) * Kp * 8);
+    lnocc::count_alloc();
+    LN_CUDA(cudaMalloc(&sl, nsl));
+    lnocc::split_ws().sl = sl;
+    lnocc::split_ws().sl_bytes = nsl;
+  }
   const lnocc::Ax one{1, 0};
   lnocc::pack(lnocc::view(A, one, one, lnocc::Ax{M, K}, one, one, lnocc::Ax{K, 1}), PA, s);
   lnocc::pack(lnocc::view(B, one, one, lnocc::Ax{N, K}, one, one, lnocc::Ax{K, 1}), PB, s);
@@ -278,6 +286,7 @@ int lnocc_debug_gemm(int precision, int M, int N, int K, const double* A, const 
   cudaFree(PB.p);
   cudaFree(dstatus);
   cudaFree(ws);
+  cudaFree(sl);
   lnocc::split_ws() = lnocc::SplitWs{};
   if (e != cudaSuccess) {
     lnocc::set_error(std::string("lnocc_debug_gemm: ") + cudaGetErrorString(e));

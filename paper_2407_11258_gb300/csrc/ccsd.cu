@@ -257,6 +257,8 @@ int Frag::build(const double* eps_in, const double* B_in) {
   scrB = alloc(scr_bytes);
   splitk_cap = 1ull << 22;
   splitk = static_cast<double*>(alloc(splitk_cap * 8));
+  slicews_bytes = slice_ws_bytes(scr_bytes);
+  slicews = alloc(slicews_bytes);
   use_workspace();
   if (oom) {
     set_error("device allocation failed in lnocc_build_ints");
@@ -304,7 +306,7 @@ int Frag::build(const double* eps_in, const double* B_in) {
       scratch_overflow = true;
     } else {
       pack(vb, PA, s);
-      gemm_f64_sym(PA, static_cast<int>(ov), out_rowmajor(ovov, ov), s);
+      gemm_f64_sym(PA, static_cast<int>(ov), out_rowmajor(ovov, ov), s, dstatus);
     }
   }
   launch_pair_L(ovov, Lpair, o, v, s);

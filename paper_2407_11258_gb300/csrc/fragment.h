@@ -31,7 +31,7 @@ struct Consts {
 
 // Sizes (bytes) of the device temporaries of one lnocc_triples call (triples.cu).
 struct TriplesPlan {
-  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, total;
+  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, slxt, slto, total;
   long long welems, nblk;
   int bc;
 };
@@ -83,7 +83,9 @@ struct Frag {
   size_t scr_bytes = 0;
   double* splitk = nullptr;  // split-K partials workspace
   size_t splitk_cap = 0;
-  void use_workspace() { split_ws() = SplitWs{splitk, splitk_cap}; }
+  void* slicews = nullptr;  // digit planes of FP64 products
+  size_t slicews_bytes = 0;
+  void use_workspace() { split_ws() = SplitWs{splitk, splitk_cap, slicews, slicews_bytes}; }
   // DIIS (subspace counters on the device: dctr[0] vectors pushed, dctr[1] vectors in use)
   int dm = 0;
   double *dvec = nullptr, *derr = nullptr, *G = nullptr, *coef = nullptr, *dpart = nullptr;

@@ -16,7 +16,9 @@
 #include <map>
 #include <mutex>
 
+#include "gemm_slices.h"
 #include "internal.h"
+#include "out_map.cuh"
 #include "ptx.cuh"
 
 namespace lnocc {
@@ -287,17 +289,6 @@ void permute(const View& v, double* dst, double beta, cudaStream_t s) {
   k_permute<<<blocks, threads, 0, s>>>(v, dst, beta);
 }
 
-__device__ __forceinline__ long long out_moff(const OutMap& C, int m) {
-  const int m0 = m % C.mdiv, mm = m / C.mdiv;
-  const int m1 = mm % C.mdiv1, m2 = mm / C.mdiv1;
-  return m2 * C.sm2 + m1 * C.sm1 + static_cast<long long>(m0) * C.sm0;
-}
-__device__ __forceinline__ long long out_noff(const OutMap& C, int n) {
-  const int n0 = n % C.ndiv, nn = n / C.ndiv;
-  const int n1 = nn % C.ndiv1, n2 = nn / C.ndiv1;
-  return n2 * C.sn2 + n1 * C.sn1 + static_cast<long long>(n0) * C.sn0;
-}
-
 __device__ __forceinline__ void store_at(const OutMap& C, long long off, double acc) {
   if (C.dst32) {
     float r = static_cast<float>(C.alpha * acc);
@@ -474,13 +465,13 @@ __global__ void __launch_bounds__(256) k_gemm_f64(const double* __restrict__ A, 
 }
 
 // Fixed-order sum of split-K partials ws[split][M][N], then the OutMap store.
-__global__ void k_splitk_reduce(const double* __restrict__ ws, int splits, int M, int N, OutMap C) {
+__global__ void k_splitk_reduce(const double* __restrict__ ws, int splits, int M, int N, OutMap C, int m0, int n0) {
   const long long total = static_cast<long long>(M) * N;
   for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<long long>(gridDim.x) * blockDim.x) {
     double acc = 0.0;
     for (int z = 0; z < splits; ++z) acc += ws[z * total + idx];
-    store_out(C, static_cast<int>(idx / N), static_cast<int>(idx % N), acc);
+    store_out(C, m0 + static_cast<int>(idx / N), n0 + static_cast<int>(idx % N), acc);
   }
 }
 
@@ -503,15 +494,22 @@ static int choose_splits(long long tiles, int nkb, long long MN) {
   return (nkb + per - 1) / per;  // no empty split
 }
 
-static void splitk_reduce(int splits, int M, int N, const OutMap& C, cudaStream_t s) {
+void splitk_reduce(int splits, int M, int N, const OutMap& C, cudaStream_t s, int m0, int n0) {
   const long long total = static_cast<long long>(M) * N;
   const int blocks = static_cast<int>(std::min<long long>((total + 255) / 256, 152LL * 8));
   count_launch();
-  k_splitk_reduce<<<blocks, 256, 0, s>>>(split_ws().p, splits, M, N, C);
+  k_splitk_reduce<<<blocks, 256, 0, s>>>(split_ws().p, splits, M, N, C, m0, n0);
 }
 
-void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s) {
+// FP64 products run on the BF16 tensor pipe (gemm_slices.cu) wherever the thread has a slice workspace; the
+// SIMT kernel serves callers that have none (lnocc_gemm_noalloc's fixed scratch). It is bound by the FP64
+// pipe (two FMA lanes per clock and SM: 1.1 TFLOP/s over the chip, and 68 us for a single 64 x 64 tile with
+// K = 64 however small the problem).
+void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s, int* dstatus) {
   (void)K;
+  if (gemm_f64_slices(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, A.Kp, C, false, 0, 0, s,
+                      dstatus))
+    return;
   const long long tiles = static_cast<long long>((N + 63) / 64) * ((M + 63) / 64);
   const int nk16 = A.Kp / 16;
   const int splits = choose_splits(tiles, nk16 / 4, static_cast<long long>(M) * N);
@@ -521,18 +519,32 @@ void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMa
   count_launch();
   k_gemm_f64<false><<<grid, 256, 0, s>>>(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, A.Kp, C,
                                   per, nsplit > 1 ? split_ws().p : nullptr, nullptr, 0);
-  if (nsplit > 1) splitk_reduce(nsplit, M, N, C, s);
+  if (nsplit > 1) splitk_reduce(nsplit, M, N, C, s, 0, 0);
 }
 
-void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s) {
+void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s, int* dstatus) {
   if (M <= 0) return;
   GemmStats& st = gemm_stats();
   st.launches++;
   st.flops += 1.0 * M * M * A.Kp;  // half of 2 M^2 K
+  const double* a = static_cast<const double*>(A.p);
+  if (gemm_f64_slices(a, a, M, M, A.Kp, C, true, 0, 0, s, dstatus)) return;
   dim3 grid((M + 63) / 64, (M + 63) / 64, 1);
   count_launch();
-  k_gemm_f64<true><<<grid, 256, 0, s>>>(static_cast<const double*>(A.p), static_cast<const double*>(A.p), M, M, A.Kp,
-                                        C, A.Kp, nullptr, nullptr, 0);
+  k_gemm_f64<true><<<grid, 256, 0, s>>>(a, a, M, M, A.Kp, C, A.Kp, nullptr, nullptr, 0);
+}
+
+void gemm_f64_lower(const Packed& A, int a_row0, int M, int N, int block, const OutMap& C, cudaStream_t s, int* dstatus) {
+  if (M <= 0 || N <= 0) return;
+  GemmStats& st = gemm_stats();
+  const double* a = static_cast<const double*>(A.p);
+  const double* a0 = a + static_cast<size_t>(a_row0) * A.Kp;
+  st.launches++;
+  st.flops += 2.0 * M * N * A.Kp;
+  if (gemm_f64_slices(a0, a, M, N, A.Kp, C, false, block, a_row0, s, dstatus)) return;
+  Packed A0 = A, B0 = A;
+  A0.p = const_cast<double*>(a0);
+  gemm_f64(A0, B0, M, N, A.Kp, C, s, dstatus);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1173,7 +1185,7 @@ __global__ void __launch_bounds__(256, 1)
   if (warp == 2) tmem_dealloc(tmem, Cfg::TMEM_COLS);
 }
 
-static int num_sms() {
+int num_sms() {
   static std::atomic<int> n{0};
   int v = n.load(std::memory_order_relaxed);
   if (v == 0) {
@@ -1203,6 +1215,15 @@ static EncodeTiledFn encode_fn() {
       fn = reinterpret_cast<EncodeTiledFn>(p);
   });
   return fn;
+}
+
+bool encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, void* base, const cuuint64_t* dims,
+                       const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle,
+                       CUtensorMapL2promotion l2) {
+  EncodeTiledFn fn = encode_fn();
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return fn && fn(map, type, rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, l2,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Operand [2][rows][Kp] bf16 as a 3-D tensor {Kp, rows, 2}; box {64, box_rows, 1}, 128-byte swizzle.
@@ -1259,7 +1280,7 @@ static void launch_tc(const Packed& A0, const Packed& B0, const Packed* A1, cons
   const int grid = static_cast<int>(std::min<long long>(ntiles, num_sms()));
   count_launch();
   k_gemm_tc<BN><<<grid, 256, Cfg::SMEM, s>>>(ta0, tb0, ta1, tb1, ta0, ta0, args);
-  if (splits > 1) splitk_reduce(splits, args.M, args.N, args.C, s);
+  if (splits > 1) splitk_reduce(splits, args.M, args.N, args.C, s, 0, 0);
 }
 
 static int heuristic_bn(int N) {
@@ -1567,6 +1588,13 @@ void gemm2_batched(const Packed& A0, const Packed& B0, const Packed* A1, const P
     TcArgs a = tc_args(maxM, N, A0.Kp / 64, A1 ? A1->Kp / 64 : 0, C, dstatus);
     a.batch = dbatch;
     dispatch_tc(A0, B0, A1, B1, a, (maxM + 127) / 128, nbatch, s);
+  } else if (A0.sl && B0.sl && (!A1 || (A1->sl && B1->sl))) {
+    gemm_sliced_batched(*A0.sl, *B0.sl, dbatch, nbatch, maxM, N, 0, C, s, dstatus);
+    if (A1) {
+      OutMap C1 = C;
+      C1.beta = 1.0;
+      gemm_sliced_batched(*A1->sl, *B1->sl, dbatch, nbatch, maxM, N, 1, C1, s, dstatus);
+    }
   } else {
     dim3 grid((maxM + 63) / 64, (N + 63) / 64, nbatch);
     count_launch();
@@ -1611,11 +1639,13 @@ void gemm_off(const Packed& A, int a_row0, const Packed& B, int b_row0, int M, i
   st.flops += 2.0 * M * N * K;
   if (A.bf16) {
     gemm_tc(A, a_row0, B, b_row0, M, N, C, s, dstatus);
+  } else if (A.sl && B.sl) {
+    gemm_sliced(*A.sl, a_row0, *B.sl, b_row0, M, N, C, s, dstatus);
   } else {
     Packed a = A, b = B;
     a.p = static_cast<double*>(A.p) + static_cast<size_t>(a_row0) * A.Kp;
     b.p = static_cast<double*>(B.p) + static_cast<size_t>(b_row0) * B.Kp;
-    gemm_f64(a, b, M, N, K, C, s);
+    gemm_f64(a, b, M, N, K, C, s, dstatus);
   }
 }
 

@@ -1,0 +1,624 @@
+// FP64 contractions on the BF16 tensor pipe.
+//
+// GB300 runs FP64 at two FMA lanes per clock and SM, a thousandth of its BF16 tensor rate, so an FP64
+// product is formed from exact BF16 products instead, after Ozaki, Ogita, Oishi and Rump (Numer.
+// Algorithms 59, 95 (2012)) and its tensor-core form (Mukunoki et al., ISC 2020):
+//   * Each operand row is cut into chunks of kChunk = 512 columns. A chunk shares one exponent E (all
+//     |x| < 2^E) and every x 2^-E becomes eight balanced radix-128 digits, x = 2^(E-6) sum_i d_i 2^(-7(i-1)),
+//     d_1..d_7 integers in [-64, 64] and the eighth the remainder rounded to BF16; plane i holds
+//     d_i 2^(-7(i-1)), exact in BF16.
+//   * A(m, :) . B(n, :) = 2^(Ea+Eb-12) sum_g S_g with S_g the digit products of i + j = g + 1. One FP32
+//     TMEM accumulator per g = 1..8. For g <= 7 every term is an integer times 2^(-7(g-1)) and
+//     |S_g| <= 7 * 512 * 64 * 64 < 2^24 units, so the accumulation is exact; accumulator 8 also takes the
+//     pairs i + j = 10 (weight 2^-56 against S_1: an FP32 rounding there is below 2^-66).
+//   * The epilogue adds the accumulators as a 72-bit integer and rounds it once to FP64.
+// What is dropped: the pairs i + j > 10 and the operands beyond their 57th bit, both relative to the
+// largest element of their chunk. The error of an element of C is about 0.05 sqrt(K) 2^-56 rowmax colmax,
+// below the K 2^-53 sum|a||b| growth of an FP64 FMA chain on the library's operands.
+// Rows whose chunk holds an infinity, a NaN, or only subnormal values are marked; their outputs are summed
+// in FP64 from the packed operand, so those propagate as in an FP64 product.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <mutex>
+
+#include "gemm_slices.h"
+#include "internal.h"
+#include "out_map.cuh"
+#include "ptx.cuh"
+
+namespace lnocc {
+namespace {
+
+constexpr int kSlices = 8;
+constexpr int kChunk = kSliceChunk;     // columns that share an exponent and an exact accumulation
+constexpr int kBadExp = 0x40000000;     // chunk that cannot be sliced
+constexpr int kBM = 128, kBN = 64, kBK = 32;
+constexpr int kABytes = kSlices * kBM * kBK * 2, kBBytes = kSlices * kBN * kBK * 2;
+constexpr int kStageBytes = kABytes + kBBytes;  // 96 KB: two stages
+constexpr int kStages = 2;
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 128 + 32 * kEpiWarps;
+constexpr int kTileBytes = kEpiWarps * 32 * 9 * 8;  // transpose tiles: 32 rows x 8 columns (+1) per warp
+constexpr int kSmem = kStages * kStageBytes + kTileBytes + 1024 + 256;
+static_assert(kSmem <= 232448, "slices pipeline does not fit shared memory");
+
+// ---------------------------------------------------------------------------------------------
+// Slicing: one warp per (row, chunk), 16 columns per lane, one read of the source.
+__global__ void __launch_bounds__(256) k_slice(const double* __restrict__ src, long long ld, int col0, int rows, int Kp,
+                                               __nv_bfloat16* __restrict__ out, long long plane, int* __restrict__ ex,
+                                               int ex_rows) {
+  const int lane = threadIdx.x % 32;
+  const int nch = (Kp + kChunk - 1) / kChunk;
+  const long long items = static_cast<long long>(rows) * nch;
+  const long long nw = static_cast<long long>(gridDim.x) * blockDim.x / 32;
+  for (long long it = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) / 32; it < items; it += nw) {
+    const int r = static_cast<int>(it / nch), ch = static_cast<int>(it % nch);
+    const int k0 = ch * kChunk, kw = min(kChunk, Kp - k0);  // kw is a multiple of 64
+    const double* s = src + r * ld + col0 + k0;
+    double2 x[8];
+    unsigned emax = 0, any = 0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int k = 2 * (lane + 32 * t);
+      x[t] = k < kw ? *reinterpret_cast<const double2*>(s + k) : make_double2(0.0, 0.0);
+      const unsigned h0 = static_cast<unsigned>(__double2hiint(x[t].x)) & 0x7fffffffu;
+      const unsigned h1 = static_cast<unsigned>(__double2hiint(x[t].y)) & 0x7fffffffu;
+      emax = max(emax, max(h0, h1));
+      any |= h0 | h1 | static_cast<unsigned>(__double2loint(x[t].x)) | static_cast<unsigned>(__double2loint(x[t].y));
+    }
+    emax = __reduce_max_sync(0xffffffffu, emax) >> 20;
+    any = __reduce_or_sync(0xffffffffu, any);
+    const bool bad = emax == 0x7ffu || (emax == 0u && any != 0u);
+    if (lane == 0) ex[static_cast<long long>(ch) * ex_rows + r] = bad ? kBadExp : static_cast<int>(emax) - 1022;
+    __nv_bfloat16* o = out + static_cast<long long>(r) * Kp + k0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int k = 2 * (lane + 32 * t);
+      if (k >= kw) break;
+      long long F[2];  // x 2^-E with 61 fraction bits
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long u = __double_as_longlong(h ? x[t].y : x[t].x);
+        const int e = static_cast<int>(u >> 52) & 0x7ff;
+        long long m = (u & 0xfffffffffffffLL) | (e > 0 ? 0x10000000000000LL : 0);
+        const int sh = static_cast<int>(emax) + 1 - max(e, 1);  // >= 1
+        m = sh <= 9 ? m << (9 - sh) : (sh < 64 ? m >> (sh - 9) : 0);
+        F[h] = bad ? 0 : (u < 0 ? -m : m);
+      }
+      float w = 1.f;
+#pragma unroll
+      for (int i = 1; i <= 7; ++i) {
+        const int sft = 62 - 7 * i;
+        float f[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const long long d = (F[h] + (1LL << (sft - 1))) >> sft;
+          F[h] -= d << sft;
+          // d in [-64, 64] to FP32 through the exponent of 1.5 2^23, scaled by the plane's weight (exact)
+          const float g = __int_as_float(0x4B400000 + static_cast<int>(d));
+          f[h] = fmaf(g, w, -12582912.f * w);
+        }
+        *reinterpret_cast<__nv_bfloat162*>(o + (i - 1) * plane + k) = __floats2bfloat162_rn(f[0], f[1]);
+        w *= 0.0078125f;
+      }
+      // |F| <= 2^12 here: the eighth plane holds F 2^-55 rounded to BF16
+      *reinterpret_cast<__nv_bfloat162*>(o + 7 * plane + k) = __floats2bfloat162_rn(
+          static_cast<float>(static_cast<int>(F[0])) * 0x1p-55f, static_cast<float>(static_cast<int>(F[1])) * 0x1p-55f);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+struct SlArgs {
+  int M, N;
+  int a_row0, b_row0;       // first rows in the sliced operands
+  int mbase, nbase;         // output row / column of local row / column 0
+  int nkb, kper;            // K blocks of 64 of this launch and per work item (kper divides 8)
+  int kblk0;                // first K block (64 columns) in the operands
+  int tiles_m, tiles_n, tiles_z;
+  int sym;                  // C = A A^T: tiles on or above the diagonal, mirrored
+  int tri, tri_row0;        // tri > 0: only columns n with n / tri <= (tri_row0 + m) / tri are needed
+  const int *ea, *eb;       // chunk exponents [chunk][rows]
+  int ea_rows, eb_rows;
+  const double *A64, *B64;  // the packed FP64 operands (rows as a_row0 / b_row0), for marked chunks
+  long long lda, ldb;
+  int asign, ashift;        // alpha = asign 2^ashift when asign != 0, else C.alpha multiplies
+  OutMap C;
+  double* ws;               // split-K partials [z][M][N], or null
+  const BatchEntry* batch;  // one problem per z
+  int seg;
+  int* status;
+};
+
+struct SlTile {
+  int m0, n0, z, M, a0, b0, kb0, nkb;
+  long long cbase;
+};
+
+// Work item t; false for an empty one (outside the problem, below the diagonal).
+__device__ __forceinline__ bool sl_tile(const SlArgs& p, int t, SlTile& ti) {
+  const int tm = t % p.tiles_m, tn = (t / p.tiles_m) % p.tiles_n;
+  ti.z = t / (p.tiles_m * p.tiles_n);
+  ti.m0 = tm * kBM;
+  ti.n0 = tn * kBN;
+  ti.M = p.M;
+  ti.a0 = p.a_row0;
+  ti.b0 = p.b_row0;
+  ti.cbase = 0;
+  ti.kb0 = ti.z * p.kper;
+  if (p.batch) {
+    const BatchEntry be = p.batch[ti.z];
+    ti.M = be.M;
+    ti.a0 = p.seg ? be.a_row1 : be.a_row0;
+    ti.b0 = p.seg ? be.b_row1 : be.b_row0;
+    ti.cbase = be.cbase;
+    ti.kb0 = 0;
+  }
+  ti.nkb = min(p.kper, p.nkb - ti.kb0);
+  ti.kb0 += p.kblk0;
+  if (p.sym && p.nbase + ti.n0 + kBN <= p.mbase + ti.m0) return false;
+  if (p.tri > 0 && (p.nbase + ti.n0) / p.tri > (p.tri_row0 + p.mbase + min(ti.m0 + kBM, p.M) - 1) / p.tri) return false;
+  return ti.m0 < ti.M && ti.nkb > 0;
+}
+
+// 32 lanes x 8 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[8][8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  // the loaded values are only defined after the wait: tie them to it
+#pragma unroll
+  for (int g = 0; g < 8; ++g)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(v[g][i]));
+}
+
+// X = hi 2^13 + lo (0 <= lo < 2^13) in units of 2^(-60): the sum of the eight accumulators.
+__device__ __forceinline__ void sl_combine(const float* a, long long& hi, int& lo) {
+  const int s1 = __float2int_rn(a[0]), s2 = __float2int_rn(a[1] * 0x1p7f), s3 = __float2int_rn(a[2] * 0x1p14f);
+  const int s4 = __float2int_rn(a[3] * 0x1p21f), s5 = __float2int_rn(a[4] * 0x1p28f), s6 = __float2int_rn(a[5] * 0x1p35f);
+  // |s1| <= 2^21, |s2| <= 2^22, ...: each pair fits 32 bits
+  const int p1 = s1 * 128 + s2, p2 = s3 * 128 + s4, p3 = s5 * 128 + s6;
+  const int t = __float2int_rn(a[6] * 0x1p48f) + __float2int_rn(a[7] * 0x1p48f);
+  hi = static_cast<long long>(p1) * (1 << 28) + (static_cast<long long>(p2) * (1 << 14) + p3) + (t >> 13);
+  lo = t & 0x1fff;
+}
+
+// (hi 2^13 + lo) 2^(e-60) rounded once to FP64; neg flips the sign.
+__device__ __forceinline__ double sl_round(long long hi, int lo, int e, bool flip) {
+  bool neg = hi < 0;
+  if (neg) {
+    hi = lo ? ~hi : -hi;
+    lo = (0x2000 - lo) & 0x1fff;
+  }
+  unsigned long long m;
+  int lz;
+  if (hi != 0) {
+    lz = __clzll(hi);
+    m = (static_cast<unsigned long long>(hi) << lz) |
+        (lz >= 13 ? static_cast<unsigned long long>(lo) << (lz - 13) : static_cast<unsigned long long>(lo) >> (13 - lz));
+  } else if (lo != 0) {
+    lz = __clzll(static_cast<long long>(lo)) + 13;
+    m = static_cast<unsigned long long>(lo) << (lz - 13);
+  } else {
+    return 0.0;
+  }
+  neg ^= flip;
+  // value = m 2^(-lz) 2^(e - 47), the top bit of m set
+  const int be = 63 - lz + e - 47 + 1023;
+  const unsigned long long f = (m >> 11) + ((m >> 10) & 1ull);
+  if (be >= 1 && be < 2046)
+    return __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(be - 1) << 52) + f) |
+                                (neg ? static_cast<long long>(0x8000000000000000ull) : 0ll));
+  const double r = ldexp(static_cast<double>(f), be - 1023 - 52);
+  return neg ? -r : r;
+}
+
+// FP64 sum over the work item's columns, for rows whose chunk could not be sliced.
+__device__ __noinline__ double sl_dot64(const double* a, const double* b, int k0, int k1) {
+  double acc = 0.0;
+  for (int k = k0; k < k1; ++k) acc = fma(a[k], b[k], acc);
+  return acc;
+}
+
+// Persistent: warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4..11 epilogue (two per
+// TMEM lane quadrant, 32 columns each). The eight accumulators of a 128 x 64 tile fill TMEM (8 x 64
+// columns, accumulator g at column 64 (g - 1)), and the eight B planes sit one after the other in shared
+// memory as 512 rows, so one MMA of N = 256 multiplies plane i of A with four planes of B into four
+// neighbouring accumulators: A is read once per four products.
+__global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__ CUtensorMap tA,
+                                                         const __grid_constant__ CUtensorMap tB, const SlArgs p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  double* tiles = reinterpret_cast<double*>(smem + kStages * kStageBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes + kTileBytes);
+  uint64_t* empty = full + kStages;
+  uint64_t* accf = empty + kStages;
+  uint64_t* acce = accf + 1;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(acce + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int ntiles = p.tiles_m * p.tiles_n * p.tiles_z;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(acce, 32 * kEpiWarps);
+    fence_barrier_init();
+    prefetch_tensormap(&tA);
+    prefetch_tensormap(&tB);
+  }
+  if (warp == 2) tmem_alloc(tmem_holder, 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+
+  if (warp == 0 && lane == 0) {
+    int g = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
+      SlTile ti;
+      if (!sl_tile(p, t, ti)) continue;
+      for (int kb = 0; kb < 2 * ti.nkb; ++kb, ++g) {
+        const int s = g % kStages;
+        if (g >= kStages && !mbar_wait(&empty[s], ((g / kStages) - 1) & 1)) {
+          atomicExch(p.status, kDevTimeoutProducer);
+          ok = false;
+          break;
+        }
+        uint8_t* st = smem + s * kStageBytes;
+        mbar_arrive_expect_tx(&full[s], kStageBytes);
+        const int kc = ti.kb0 * 64 + kb * kBK;
+        tma_load_3d(st, &tA, &full[s], kc, ti.a0 + ti.m0, 0);
+        tma_load_3d(st + kABytes, &tB, &full[s], kc, ti.b0 + ti.n0, 0);
+      }
+    }
+    for (int q = (g > kStages ? g - kStages : 0); q < g; ++q) mbar_wait(&full[q % kStages], (q / kStages) & 1);
+  } else if (warp == 1 && lane == 0) {
+    int g = 0, it = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
+      SlTile ti;
+      if (!sl_tile(p, t, ti)) continue;
+      if (it > 0 && !mbar_wait(acce, (it - 1) & 1)) {
+        atomicExch(p.status, kDevTimeoutMma);
+        break;
+      }
+      tc_fence_after();
+      for (int kb = 0; kb < 2 * ti.nkb; ++kb, ++g) {
+        const int s = g % kStages;
+        if (!mbar_wait(&full[s], (g / kStages) & 1)) {
+          atomicExch(p.status, kDevTimeoutMma);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t a0 = smem_u32(smem + s * kStageBytes), b0 = a0 + kABytes;
+#pragma unroll
+        for (int kk = 0; kk < kBK / 16; ++kk) {
+          const uint32_t off = kk * 32;
+          const uint32_t first = (kb | kk) != 0 ? 1u : 0u;
+#pragma unroll
+          for (int i = 0; i < kSlices; ++i) {
+            // plane i of A against planes 0 .. 7 - i of B: accumulators i .. 7
+            const uint64_t da = sdesc_sw64(a0 + i * (kBM * kBK * 2) + off);
+#pragma unroll
+            for (int j = 0; j < kSlices - i; j += 4) {
+              const int nj = kSlices - i - j < 4 ? kSlices - i - j : 4;
+              mma_bf16(tmem + (i + j) * kBN, da, sdesc_sw64(b0 + j * (kBN * kBK * 2) + off),
+                       idesc_bf16_f32(kBM, nj * kBN), i == 0 ? first : 1u);
+            }
+            // and plane 8 - i: the leading dropped diagonal, into accumulator 7
+            if (i > 0)
+              mma_bf16(tmem + 7 * kBN, da, sdesc_sw64(b0 + (8 - i) * (kBN * kBK * 2) + off),
+                       idesc_bf16_f32(kBM, kBN), 1u);
+          }
+        }
+        mma_commit(&empty[s]);
+      }
+      mma_commit(accf);
+      ++it;
+    }
+  } else if (warp >= 4) {
+    const int ew = warp - 4, quad = ew & 3, half = ew >> 2;
+    double* tile = tiles + ew * (32 * 9);
+    const OutMap C = p.ws ? OutMap{p.ws, 0, p.N, 0, 1, 1 << 30, 1 << 30, 1.0, 0.0} : p.C;
+    const int mb = p.ws ? 0 : p.mbase, nb = p.ws ? 0 : p.nbase;  // split-K partials are local
+    const bool colc = !p.sym && C.sn0 == 1 && !C.dst32;  // columns contiguous: stores go through the transpose tile
+    const bool flip = !p.ws && p.asign < 0;
+    const int ash = p.ws ? 0 : p.ashift;
+    const bool mul = !p.ws && p.asign == 0;
+    int it = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      SlTile ti;
+      if (!sl_tile(p, t, ti)) continue;
+      if (!mbar_wait(accf, it & 1)) {
+        if (lane == 0) atomicExch(p.status, kDevTimeoutEpilogue);
+        break;
+      }
+      ++it;
+      tc_fence_after();
+      const int m = ti.m0 + quad * 32 + lane, nbase = ti.n0 + half * 32;
+      const bool mok = m < ti.M;
+      const int ch = ti.kb0 / (kChunk / 64);
+      const int ea = mok ? p.ea[static_cast<long long>(ch) * p.ea_rows + ti.a0 + m] : 0;
+      const long long cb = ti.cbase + (p.ws ? static_cast<long long>(ti.z) * p.M * p.N : 0);
+      const long long moff = mok ? out_moff(C, mb + m) : 0;
+      long long roff[8];  // destination rows of the transposed stores
+      if (colc) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int mm = ti.m0 + quad * 32 + 4 * q + lane / 8;
+          roff[q] = mm < ti.M ? cb + out_moff(C, mb + mm) : -1;
+        }
+      }
+      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * 32;
+#pragma unroll 1
+      for (int c8 = 0; c8 < 4; ++c8) {
+        float v[8][8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) tmem_ld8(acc + g * kBN + 8 * c8, v[g]);
+        tmem_wait_ld(v);
+        if (c8 == 3) {  // everything read: the next tile's products may start
+          tc_fence_before();
+          mbar_arrive(acce);
+        }
+        const int n0 = nbase + 8 * c8;
+        if (n0 >= p.N) continue;
+        double r[8];
+        // lane j < 8 holds the exponent of column n0 + j
+        const int nl = n0 + (lane & 7);
+        const int ebl = nl < p.N ? p.eb[static_cast<long long>(ch) * p.eb_rows + ti.b0 + nl] : 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int n = n0 + j;
+          const int eb = __shfl_sync(0xffffffffu, ebl, j);
+          float a[8];
+#pragma unroll
+          for (int g = 0; g < 8; ++g) a[g] = v[g][j];
+          long long hi;
+          int lo;
+          sl_combine(a, hi, lo);
+          if (ea == kBadExp || eb == kBadExp) {
+            r[j] = 0.0;
+            if (mok && n < p.N) {
+              const double x = sl_dot64(p.A64 + (ti.a0 + m) * p.lda, p.B64 + (ti.b0 + n) * p.ldb, ti.kb0 * 64,
+                                        (ti.kb0 + ti.nkb) * 64);
+              r[j] = p.ws ? x : C.alpha * x;
+            }
+          } else {
+            r[j] = sl_round(hi, lo, ea + eb + ash, flip);
+            if (mul) r[j] *= C.alpha;
+          }
+        }
+        auto put = [&](long long off, double x) {
+          if (C.dst32) {
+            float y = static_cast<float>(x);
+            if (C.beta != 0.0) y += static_cast<float>(C.beta) * C.dst32[off];
+            C.dst32[off] = y;
+          } else if (C.beta == 0.0) {
+            C.dst[off] = x;
+          } else if (C.beta == 1.0) {
+            asm volatile("red.global.add.f64 [%0], %1;" ::"l"(C.dst + off), "d"(x) : "memory");
+          } else {
+            C.dst[off] = x + C.beta * C.dst[off];
+          }
+        };
+        if (colc) {
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 8; ++j) tile[lane * 9 + j] = r[j];
+          __syncwarp();
+          const int n = n0 + (lane & 7);
+          if (n < p.N) {
+            const long long noff = out_noff(C, nb + n);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              if (roff[q] >= 0) put(roff[q] + noff, tile[(4 * q + lane / 8) * 9 + (lane & 7)]);
+          }
+        } else if (mok) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int n = n0 + j;
+            if (n >= p.N || (p.sym && nb + n < mb + m)) continue;
+            put(cb + moff + out_noff(C, nb + n), r[j]);
+            if (p.sym && nb + n > mb + m) put(cb + out_moff(C, nb + n) + out_noff(C, mb + m), r[j]);
+          }
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 2) tmem_dealloc(tmem, 512);
+}
+
+bool make_slice_map(CUtensorMap* map, const void* p, long long rows, int Kp, int box_rows) {
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(Kp), static_cast<cuuint64_t>(rows), kSlices};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(Kp) * 2, static_cast<cuuint64_t>(Kp) * 2 * static_cast<cuuint64_t>(rows)};
+  cuuint32_t box[3] = {kBK, static_cast<cuuint32_t>(box_rows), kSlices};
+  return encode_tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(p), dims, strides, box,
+                           CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+}
+
+void launch_sl(const Sliced& A, const Sliced& B, SlArgs a, cudaStream_t s) {
+  static std::once_flag once;
+  std::call_once(once, [] { cudaFuncSetAttribute(k_gemm_sl, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem); });
+  CUtensorMap ta, tb;
+  if (!make_slice_map(&ta, A.p, A.rows, A.Kp, kBM) || !make_slice_map(&tb, B.p, B.rows, B.Kp, kBN)) {
+    set_error("cuTensorMapEncodeTiled failed (slices)");
+    return;
+  }
+  a.ea = A.ex;
+  a.eb = B.ex;
+  a.ea_rows = A.rows;
+  a.eb_rows = B.rows;
+  a.A64 = A.src;
+  a.B64 = B.src;
+  a.lda = A.ld;
+  a.ldb = B.ld;
+  int e = 0;
+  const double f = std::frexp(a.C.alpha, &e);
+  a.asign = f == 0.5 ? 1 : f == -0.5 ? -1 : 0;
+  a.ashift = a.asign ? e - 1 : 0;
+  const long long n = static_cast<long long>(a.tiles_m) * a.tiles_n * a.tiles_z;
+  const int grid = static_cast<int>(std::min<long long>(n, num_sms()));
+  count_launch();
+  k_gemm_sl<<<grid, kThreads, kSmem, s>>>(ta, tb, a);
+}
+
+}  // namespace
+
+size_t slice_bytes(long long rows, int Kp) {
+  const size_t planes = static_cast<size_t>(rows) * Kp * 2 * kSlices;
+  const size_t ex = static_cast<size_t>(rows) * ((Kp + kChunk - 1) / kChunk) * 4;
+  return (planes + 255) / 256 * 256 + (ex + 255) / 256 * 256;
+}
+
+Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long ld) {
+  Sliced s;
+  s.rows = static_cast<int>(rows);
+  s.Kp = Kp;
+  s.p = mem;
+  s.ex = reinterpret_cast<int*>(static_cast<unsigned char*>(mem) +
+                                (static_cast<size_t>(rows) * Kp * 2 * kSlices + 255) / 256 * 256);
+  s.src = src;
+  s.ld = ld;
+  return s;
+}
+
+void slice(const Sliced& d, cudaStream_t s) {
+  if (d.rows <= 0) return;
+  const long long items = static_cast<long long>(d.rows) * ((d.Kp + kChunk - 1) / kChunk);
+  const int blocks = static_cast<int>(std::min<long long>((items + 7) / 8, 152LL * 16));
+  count_launch();
+  k_slice<<<blocks, 256, 0, s>>>(d.src, d.ld, 0, d.rows, d.Kp, static_cast<__nv_bfloat16*>(d.p),
+                                 static_cast<long long>(d.rows) * d.Kp, d.ex, d.rows);
+}
+
+// One product of sliced operands (rows from a_row0 / b_row0), K in launches of one chunk unless the
+// partials of several fit the split-K workspace.
+static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C,
+                             int mbase, int nbase, const BatchEntry* batch, int nbatch, int seg, int sym, int tri,
+                             int tri_row0, cudaStream_t s, int* dstatus) {
+  SlArgs a{};
+  a.M = M;
+  a.N = N;
+  a.a_row0 = a_row0;
+  a.b_row0 = b_row0;
+  a.mbase = mbase;
+  a.nbase = nbase;
+  a.tiles_m = (M + kBM - 1) / kBM;
+  a.tiles_n = (N + kBN - 1) / kBN;
+  a.sym = sym;
+  a.tri = tri;
+  a.tri_row0 = tri_row0;
+  a.C = C;
+  a.batch = batch;
+  a.seg = seg;
+  a.status = dstatus;
+  const int nkb = A.Kp / 64;
+  const long long tiles = static_cast<long long>(a.tiles_m) * a.tiles_n, MN = static_cast<long long>(M) * N;
+  constexpr int kcb = kChunk / 64;
+  if (!batch && !sym) {
+    // split K over work items while they do not fill the SMs (a tile of 512 columns takes some 28 us of
+    // MMAs, 64 columns 3.6 us), the FP64 partials summed by the fixed-order reduction
+    const SplitWs& w = split_ws();
+    int kper = kcb;
+    while (kper > 1 && tiles * ((nkb + kper - 1) / kper) < num_sms()) kper /= 2;
+    auto fits = [&](int k) { return w.p && static_cast<size_t>((nkb + k - 1) / k) * static_cast<size_t>(MN) <= w.cap; };
+    while (kper < kcb && !fits(kper)) kper *= 2;
+    const int z = (nkb + kper - 1) / kper;
+    if (z > 1 && fits(kper)) {
+      a.nkb = nkb;
+      a.kper = kper;
+      a.tiles_z = z;
+      a.ws = w.p;
+      launch_sl(A, B, a, s);
+      splitk_reduce(z, M, N, C, s, mbase, nbase);
+      return;
+    }
+  }
+  for (int k0 = 0; k0 < nkb; k0 += kcb) {
+    a.kblk0 = k0;
+    a.nkb = std::min(kcb, nkb - k0);
+    a.kper = kcb;
+    a.tiles_z = batch ? nbatch : 1;
+    launch_sl(A, B, a, s);
+    a.C.beta = 1.0;
+  }
+}
+
+void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C, cudaStream_t s,
+                 int* dstatus) {
+  gemm_sliced_rows(A, a_row0, B, b_row0, M, N, C, 0, 0, nullptr, 1, 0, 0, 0, 0, s, dstatus);
+}
+
+void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int seg,
+                         const OutMap& C, cudaStream_t s, int* dstatus) {
+  gemm_sliced_rows(A, 0, B, 0, maxM, N, C, 0, 0, dbatch, nbatch, seg, 0, 0, 0, s, dstatus);
+}
+
+// A (M rows) and B (N rows) packed FP64, K = Kp: slices panels of both into the slice workspace.
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, const OutMap& C, bool sym, int tri,
+                     int tri_row0, cudaStream_t s, int* dstatus) {
+  const SplitWs& w = split_ws();
+  if (!w.sl || !dstatus) return false;
+  auto bytes = [](long long rows, int k) { return slice_bytes(rows, k); };
+  if (bytes(std::min(M, 512), std::min(Kp, 2 * kChunk)) + bytes(std::min(N, 256), std::min(Kp, 2 * kChunk)) > w.sl_bytes)
+    return false;
+  unsigned char* base = static_cast<unsigned char*>(w.sl);
+  const bool same = A == B && M == N;
+  if (same && bytes(M, Kp) <= w.sl_bytes) {
+    const Sliced SA = slice_at(base, M, Kp, A, Kp);
+    slice(SA, s);
+    gemm_sliced_rows(SA, 0, SA, 0, M, N, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+    return true;
+  }
+  // the K panel is the whole of K unless even a few row tiles of it would not fit
+  int kp = Kp;
+  while (kp > 2 * kChunk && bytes(std::min(M, 512), kp) + bytes(std::min(N, 256), kp) > w.sl_bytes)
+    kp = (kp / 2 + kChunk - 1) / kChunk * kChunk;
+  OutMap Ck = C;
+  for (int k0 = 0; k0 < Kp; k0 += kp) {
+    const int kw = std::min(kp, Kp - k0);
+    // B whole when it leaves room for a quarter of the workspace, else panels of half of it
+    const size_t rb = bytes(64, kw);
+    int nb = N;
+    if (bytes(N, kw) > w.sl_bytes / 4 * 3 && bytes(N, kw) + bytes(M, kw) > w.sl_bytes)
+      nb = std::max(64, static_cast<int>(w.sl_bytes / 2 / rb) * 64);
+    for (int n0 = 0; n0 < N; n0 += nb) {
+      const int nn = std::min(nb, N - n0);
+      const Sliced SB = slice_at(base, nn, kw, B + static_cast<size_t>(n0) * Kp + k0, Kp);
+      const size_t used = bytes(nn, kw), room = w.sl_bytes - used;
+      int mb = M;
+      if (bytes(M, kw) > room) mb = std::max(128, static_cast<int>(room / bytes(128, kw)) * 128);
+      slice(SB, s);
+      for (int m0 = 0; m0 < M; m0 += mb) {
+        const int mm = std::min(mb, M - m0);
+        if (sym && n0 + nn <= m0) continue;
+        const Sliced SA = slice_at(base + used, mm, kw, A + static_cast<size_t>(m0) * Kp + k0, Kp);
+        slice(SA, s);
+        gemm_sliced_rows(SA, 0, SB, 0, mm, nn, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+      }
+    }
+    Ck.beta = 1.0;
+  }
+  return true;
+}
+
+}  // namespace lnocc

@@ -1,0 +1,34 @@
+// FP64 contractions on the BF16 tensor pipe (gemm_slices.cu): operands cut into BF16 digit planes.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "internal.h"
+
+namespace lnocc {
+
+constexpr int kSliceChunk = 512;  // columns that share one exponent
+
+// Rows of a packed FP64 operand (row stride ld, Kp columns) as eight BF16 planes [8][rows][Kp] and the
+// exponents [ceil(Kp / 512)][rows] of their chunks.
+struct Sliced {
+  void* p = nullptr;
+  int* ex = nullptr;
+  int rows = 0, Kp = 0;
+  const double* src = nullptr;
+  long long ld = 0;
+};
+
+size_t slice_bytes(long long rows, int Kp);  // device bytes of one Sliced operand
+Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long ld);
+void slice(const Sliced& d, cudaStream_t s);  // fill the planes from src
+void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C, cudaStream_t s,
+                 int* dstatus);
+void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int seg,
+                         const OutMap& C, cudaStream_t s, int* dstatus);
+// C = A B^T for packed FP64 operands through the thread's slice workspace (split_ws().sl): false when
+// there is none (or it is too small): the caller then runs the FP64 SIMT kernel. sym: A == B, the upper
+// part computed and mirrored. tri > 0: only elements with n / tri <= (tri_row0 + m) / tri are needed.
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, const OutMap& C, bool sym, int tri,
+                     int tri_row0, cudaStream_t s, int* dstatus);
+
+}  // namespace lnocc

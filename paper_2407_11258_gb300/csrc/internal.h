@@ -1,6 +1,7 @@
 // Internal (host-side) interfaces shared by the translation units of liblnocc.
 #pragma once
 #include <atomic>
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -67,11 +68,15 @@ inline View view(const double* p, Ax r2, Ax r1, Ax r0, Ax k2, Ax k1, Ax k0, doub
 }
 constexpr Ax kOne{1, 0};
 
-// A packed operand: FP64 [rows][Kp] or BF16 [2][rows][Kp] (hi plane, lo plane).
+struct Sliced;  // gemm_slices.h
+
+// A packed operand: FP64 [rows][Kp] or BF16 [2][rows][Kp] (hi plane, lo plane). An FP64 operand that
+// many products read may carry its digit planes (sl).
 struct Packed {
   void* p = nullptr;
   int rows = 0, Kp = 0;
   bool bf16 = false;
+  const Sliced* sl = nullptr;
 };
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -82,9 +87,12 @@ void pack_rows(const View& v, Packed& full, int row0, cudaStream_t s);
 void pack_cols(const View& v, Packed& full, int row0, int col0, int width, cudaStream_t s);
 // dst[r*K + k] = view(r, k) + beta * dst[r*K + k]   (FP64, no padding)
 void permute(const View& v, double* dst, double beta, cudaStream_t s);
-void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s);
+void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s, int* dstatus);
 // C = A A^T in FP64 with the symmetric half computed once and mirrored (A FP64-packed, M rows)
-void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s);
+void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s, int* dstatus);
+// Rows [a_row0, a_row0 + M) of A against rows [0, N) of A in FP64; only elements whose column block
+// n / block does not exceed the row block (a_row0 + m) / block are needed (others may be left unset).
+void gemm_f64_lower(const Packed& A, int a_row0, int M, int N, int block, const OutMap& C, cudaStream_t s, int* dstatus);
 void gemm_tc(const Packed& A, int a_row0, const Packed& B, int b_row0, int M, int N, const OutMap& C,
              cudaStream_t s, int* dstatus);
 // rows [a_row0, a_row0 + M) of A against rows [b_row0, b_row0 + N) of B
@@ -120,13 +128,28 @@ struct GrpSpec {
 void gemm_grouped(const Packed* const ops[4], const int box_rows[4], const GrpSpec& g, const OutMap* Cg, int ncg,
                   cudaStream_t s, int* dstatus);
 
-// Workspace for split-K partials (FP64 elements), provided by the caller of the contraction engine.
-// Per host thread: each thread drives its own fragment and stream.
+// Workspaces of the contraction engine, provided by its caller: split-K partials (p, cap FP64 elements)
+// and the digit planes of FP64 products (sl, sl_bytes). Per host thread: each thread drives its own
+// fragment and stream.
 struct SplitWs {
   double* p = nullptr;
   size_t cap = 0;
+  void* sl = nullptr;
+  size_t sl_bytes = 0;
 };
 SplitWs& split_ws();
+// Bytes of a slice workspace for products whose operands take at most `operand_bytes` packed in FP64: room
+// for the planes of both (16 bytes an element) up to 256 MB (panels beyond that).
+inline size_t slice_ws_bytes(size_t operand_bytes) {
+  const size_t want = 4 * operand_bytes + (size_t(1) << 20);
+  return want < (size_t(256) << 20) ? want : size_t(256) << 20;
+}
+// Fixed-order sum of split-K partials (split_ws().p) into C, output rows / columns from m0 / n0.
+void splitk_reduce(int splits, int M, int N, const OutMap& C, cudaStream_t s, int m0, int n0);
+int num_sms();
+bool encode_tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, void* base, const cuuint64_t* dims,
+                       const cuuint64_t* strides, const cuuint32_t* box, CUtensorMapSwizzle swizzle,
+                       CUtensorMapL2promotion l2);
 
 struct GemmStats {
   long long launches = 0;

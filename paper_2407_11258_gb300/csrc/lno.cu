@@ -307,11 +307,17 @@ int finish(cudaStream_t s, int* dstatus, const char* who) {
   return LNOCC_OK;
 }
 
-struct SplitScope {  // split-K partials for long-K / small-output contractions, for the call's duration
+struct SplitScope {  // split-K partials and FP64 digit planes, for the call's duration
   SplitWs saved;
-  SplitScope(Arena& ar) : saved(split_ws()) {
+  // operand_bytes: the largest FP64-packed operand of the call (0: no FP64 products)
+  SplitScope(Arena& ar, size_t operand_bytes) : saved(split_ws()) {
     double* ws = ar.get_n<double>(1LL << 22);
     split_ws() = ws ? SplitWs{ws, size_t(1) << 22} : SplitWs{};
+    if (operand_bytes > 0) {
+      const size_t n = slice_ws_bytes(operand_bytes);
+      split_ws().sl = ar.get(n);
+      split_ws().sl_bytes = split_ws().sl ? n : 0;
+    }
   }
   ~SplitScope() { split_ws() = saved; }
 };
@@ -407,7 +413,8 @@ extern "C" int lnocc_lno_densities(int precision, int kind, int nocc, int nvir, 
     return LNOCC_ENOMEM;
   }
   LN_CUDA(cudaMemsetAsync(dstatus, 0, 16, s));
-  SplitScope split(ar);
+  const long long kpo = round_up(N, 64), kpd = static_cast<long long>(v) * round_up(static_cast<int>(std::min(ov, 1LL << 30)), 64);
+  SplitScope split(ar, bf ? 0 : static_cast<size_t>(std::max(ov * kpo, kpd)) * 8);
   Engine eng{ar, bf, s, dstatus};
   count_launch(2);
   k_zero<<<grid1(1LL * o * o), 256, 0, s>>>(D_occ, 1LL * o * o);
@@ -604,7 +611,7 @@ extern "C" int lnocc_active_space(int precision, int nocc, int nvir, int naux, c
   k_rotate_cols<<<grid1(1LL * o * no_F), 256, 0, s>>>(C_occ, o, no_F, Ro, oo_, Co, no_F);
   k_rotate_cols<<<grid1(1LL * v * nv_F), 256, 0, s>>>(C_vir, v, nv_F, Rv, ov_, Cv, nv_F);
   k_block_diag<<<grid1(1LL * n * nF), 256, 0, s>>>(Co, o, no_F, Cv, v, nv_F, CF);
-  SplitScope split(ar);
+  SplitScope split(ar, precision == LNOCC_PREC_MIXED ? 0 : static_cast<size_t>(nq_h) * n * round_up(n, 64) * 8);
   Engine eng{ar, precision == LNOCC_PREC_MIXED, s, dstatus};
   // per block of auxiliary indices Q (bounded packed operands):
   // H[Q][p][t] = sum_q B[Q][p][q] C_F[q][t]: rows (Q, p), K q; columns t (rows of C_F^T)

@@ -95,7 +95,7 @@ __global__ void k_mp2_sum(const double* __restrict__ part, long long n, double* 
 }
 
 struct Mp2Plan {
-  size_t status, packed, X, part, total;
+  size_t status, packed, X, part, slices, total;
   int ni;
 };
 
@@ -113,7 +113,8 @@ Mp2Plan mp2_plan(bool bf, int o, int v, int N) {
   p.packed = align256(ov * Kp * (bf ? 4 : 8));
   p.X = align256(static_cast<size_t>(p.ni) * row_bytes);
   p.part = align256(static_cast<size_t>(T) * (T + 1) / 2 * o * p.ni * 8 + 8);
-  p.total = p.status + p.packed + p.X + p.part;
+  p.slices = bf ? 0 : align256(slice_ws_bytes(p.packed / 2));  // digit planes of B_ov (up to 256 MB)
+  p.total = p.status + p.packed + p.X + p.part + p.slices;
   return p;
 }
 
@@ -180,11 +181,18 @@ extern "C" int lnocc_mp2_energy(int precision, int nocc, int nvir, int naux, con
     pack(view(B_ov, kOne, Ax{o, v}, Ax{v, 1}, kOne, kOne, Ax{N, ov}), PA, s);
     const SplitWs saved = split_ws();
     split_ws() = SplitWs{};  // no split-K: its partials would need workspace beyond the plan
+    if (plan.slices > 0) {
+      split_ws().sl = base + plan.status + plan.packed + plan.X + plan.part;
+      split_ws().sl_bytes = plan.slices;
+    }
     const int T = (v + kTile - 1) / kTile;
     for (int i0 = 0; i0 < o; i0 += plan.ni) {
       const int ni = std::min(plan.ni, o - i0);
       const int ncols = (i0 + ni) * v;  // pairs j <= i only
-      gemm_off(PA, i0 * v, PA, 0, ni * v, ncols, N, out_rowmajor(X, ncols), s, dstatus);
+      if (bf)
+        gemm_off(PA, i0 * v, PA, 0, ni * v, ncols, N, out_rowmajor(X, ncols), s, dstatus);
+      else  // pairs j > i are not read: their tiles are skipped
+        gemm_f64_lower(PA, i0 * v, ni * v, ncols, v, out_rowmajor(X, ncols), s, dstatus);
       dim3 grid(T * (T + 1) / 2, i0 + ni, ni);
       count_launch(2);
       k_mp2_pairs<<<grid, 256, 0, s>>>(X, ncols, i0, ni, o, v, eps, part);

@@ -29,6 +29,7 @@
 
 #include "ccsd_kernels.h"
 #include "fragment.h"
+#include "gemm_slices.h"
 #include "internal.h"
 
 namespace lnocc {
@@ -923,7 +924,17 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
   p.u = static_cast<size_t>(o) * 8 * 8;  // U padded to at most 8 LOs
   p.ovt = bf ? static_cast<size_t>(vv * oo) * 4 : 0;  // FP32 (ia|jb) in block-energy order (mixed)
   auto al = [](size_t x) { return (std::max<size_t>(x, 256) + 255) / 256 * 256; };
-  p.total = 2 * al(p.xt) + 2 * al(p.to) + al(p.ovoo) + al(p.pbvv) + al(p.ovvv_chunk) + al(p.w) + al(p.tpart) +
+  // FP64: the digit planes of the four operands, cut once per call instead of in every product that reads
+  // them; beyond 32 GB (nocc 24 with nvir above 270) the products run on the SIMT kernel from the packed
+  // operands alone
+  const int Ktp = round_up(Kt, 64);
+  const size_t slxt = slice_bytes(vv * o, Ktp), slto = slice_bytes(v * oo, Ktp);
+  if (!bf && 2 * (slxt + slto) <= (size_t(32) << 30)) {
+    p.slxt = slxt;
+    p.slto = slto;
+    p.total += 2 * al(p.slxt) + 2 * al(p.slto);
+  }
+  p.total += 2 * al(p.xt) + 2 * al(p.to) + al(p.ovoo) + al(p.pbvv) + al(p.ovvv_chunk) + al(p.w) + al(p.tpart) +
             2 * al(p.batch) + al(p.u) + (bf ? al(p.ovt) : 0);
   return p;
 }
@@ -1059,6 +1070,22 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   // XT2[c][a][k][v + l] = -t_kl^ca (the l-terms enter W with a minus sign)
   pack_cols(view(t2, A_(v, 1), A_(v, v), A_(o, o * vv), kOne, kOne, A_(o, vv), -1.0), XT1, 0, v, wl, s);
   pack_cols(view(t2, A_(v, v), A_(v, 1), A_(o, o * vv), kOne, kOne, A_(o, vv), -1.0), XT2, 0, v, wl, s);
+
+  Sliced sls[4];
+  if (tp.slxt > 0) {
+    Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
+    for (int k = 0; k < 4; ++k) {
+      void* mem = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
+      if (!mem) {
+        cleanup();
+        set_error("lnocc_triples: device allocation failed (digit planes)");
+        return LNOCC_ENOMEM;
+      }
+      sls[k] = slice_at(mem, ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
+      slice(sls[k], s);
+      ops[k]->sl = &sls[k];
+    }
+  }
 
   // ---- slabs of fixed b: virtual c in [b, v) in chunks, a in [0, b]; W_chunk[c - c0][a][i][j][k]
   const size_t wsz = bf ? 4 : 8;
