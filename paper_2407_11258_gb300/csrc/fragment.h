@@ -31,7 +31,7 @@ struct Consts {
 
 // Sizes (bytes) of the device temporaries of one lnocc_triples call (triples.cu).
 struct TriplesPlan {
-  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, slxt, slto, total;
+  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, tri, slxt, slto, total;
   long long welems, nblk;
   int bc;
 };

@@ -31,6 +31,7 @@
 #include "fragment.h"
 #include "gemm_slices.h"
 #include "internal.h"
+#include "triples_energy.h"
 
 namespace lnocc {
 
@@ -40,55 +41,6 @@ namespace {
 
 // Position permutations of three slots, listed as (p1, p2, p3) in 0-based slots.
 __constant__ int kPerm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-
-// Compensated FP32 summation for the FP32 block-energy kernels: a running sum s and the sum c of the
-// rounding errors of its additions, each error obtained exactly by Knuth's TwoSum (TAOCP vol. 2,
-// 4.2.2), cascaded as in the Sum2 algorithm of Ogita, Rump and Oishi (SIAM J. Sci. Comput. 26, 1955
-// (2005)). s + c is as accurate as a sum formed in twice the FP32 precision (error about
-// u|S| + (n u)^2 sum|x_i|, u = 2^-24), which keeps the block partials as accurate as the FP64 sums
-// they replace without FP64-pipe work (the part's FP64 rate is a small fraction of its FP32 rate).
-// The _rn intrinsics keep the compiler from fusing or reordering the error terms.
-struct CSum {
-  float s, c;
-};
-__device__ __forceinline__ void csum_add(CSum& a, float x) {
-  const float t = __fadd_rn(a.s, x);
-  const float bp = __fsub_rn(t, a.s);
-  const float err = __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, bp)), __fsub_rn(x, bp));
-  a.s = t;
-  a.c = __fadd_rn(a.c, err);
-}
-__device__ __forceinline__ void csum_merge(CSum& a, const CSum& b) {
-  csum_add(a, b.s);
-  a.c = __fadd_rn(a.c, b.c);
-}
-// Block result {canonical, projected} of two compensated sums: warp trees, then warp 0 over the warps'
-// sums, in a fixed order; thread 0 writes -(s + c) / 3 in FP64 (the 1/3 of the six orderings).
-__device__ __forceinline__ void csum_block_out(CSum e0, CSum e1, double* out, long long blk_id) {
-  __shared__ float4 sh[32];
-  for (int off = 16; off > 0; off >>= 1) {
-    CSum o0, o1;
-    o0.s = __shfl_xor_sync(0xffffffffu, e0.s, off);
-    o0.c = __shfl_xor_sync(0xffffffffu, e0.c, off);
-    o1.s = __shfl_xor_sync(0xffffffffu, e1.s, off);
-    o1.c = __shfl_xor_sync(0xffffffffu, e1.c, off);
-    csum_merge(e0, o0);
-    csum_merge(e1, o1);
-  }
-  const int w = threadIdx.x / 32, l = threadIdx.x % 32;
-  if (l == 0) sh[w] = make_float4(e0.s, e0.c, e1.s, e1.c);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    CSum a0{0.f, 0.f}, a1{0.f, 0.f};
-    for (int q = 0; q < static_cast<int>(blockDim.x / 32); ++q) {
-      const float4 t = sh[q];
-      csum_merge(a0, CSum{t.x, t.y});
-      csum_merge(a1, CSum{t.z, t.w});
-    }
-    out[2 * blk_id] = -(static_cast<double>(a0.s) + static_cast<double>(a0.c)) / 3.0;
-    out[2 * blk_id + 1] = -(static_cast<double>(a1.s) + static_cast<double>(a1.c)) / 3.0;
-  }
-}
 
 // Block energy, generic form: one CTA per (pair, a) with a <= b; threads over (j, k). Any nocc and any
 // number of LOs: the projected i-sums are kept for up to kLoChunk LOs at a time, and for more LOs the
@@ -199,8 +151,7 @@ __global__ void k_t_energy(const TW* __restrict__ W, long long slot_stride, int 
 // and every distinct ordering of (a, b, c); the i-sums are accumulated in Real and the block sum in FP64.
 // VFLY: only w is staged and v = w + disc s is recomputed where it is read (the slices, t1 columns and
 // d_m are in shared memory already); half the shared memory, for blocks too large to stage both.
-// Launched for the FP64 path; the mixed path runs k_t_energy_f32 (w and v staged) or k_t_energy_vfly
-// (w staged) below.
+// Launched for the FP64 path; the mixed path runs k_t_energy_pair or k_t_energy_single below.
 template <typename TW, typename Real, int NLO, bool VFLY>
 __global__ void k_t_energy_staged(const TW* __restrict__ W, long long slot_stride, int b, int c0, int o, int v,
                                   const double* __restrict__ eps, const double* __restrict__ t1,
@@ -373,408 +324,25 @@ __global__ void k_t_energy_staged(const TW* __restrict__ W, long long slot_strid
   }
 }
 
-// Block energy of the mixed path with w and v both staged (FP32 W): the same quantities and orderings
-// as k_t_energy_staged with Real = float and both w and v staged (the form it replaced on this path),
-// with the data movement reworked and the partials across (j, k) summed in compensated FP32 (CSum)
-// instead of FP64:
-//  * the staging pass issues eight independent W loads per thread before it uses any of them;
-//  * w and v of one (y0, y1, y2) sit side by side, so a placement is one 8-byte shared-memory load;
-//  * the projected i-sums of z and y for one LO form a pair updated by one packed FP32 FMA, with
-//    U[i][alpha] duplicated into both halves of a pair in shared memory.
-// OC > 0: compiled for nocc = OC (constant strides and trip counts); OC = 0: any nocc (o_in).
-template <int NLO, int OC>
-__global__ void __launch_bounds__(256, NLO <= 2 ? 4 : 2)
-    k_t_energy_f32(const float* __restrict__ W, long long slot_stride, int b, int c0, int o_in, int v,
-                   const double* __restrict__ eps, const double* __restrict__ t1, const float* __restrict__ ovT,
-                   const double* __restrict__ U, double* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int o = OC > 0 ? OC : o_in;
-  const int slot = blockIdx.y, a = blockIdx.x;
-  const int c = c0 + slot;
-  const long long blk_id = static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x;
-  const int o2 = o * o, o3 = o2 * o;
-  const int S1 = o + 1, S0 = o * S1 + 1;  // padded strides of the staged block (odd for even o)
-  const int blk = o * S0;
-  float2* swv = reinterpret_cast<float2*>(smraw);  // (w, v) at y0 * S0 + y1 * S1 + y2
-  float* fs = reinterpret_cast<float*>(smraw) + 2 * blk;
-  const int P1 = o + 1, o2p = o * P1;
-  float* Sab = fs;  // (y0 a|y1 b)
-  float* Sac = Sab + o2p;
-  float* Sbc = Sac + o2p;
-  float* ta = Sbc + o2p;
-  float* tb = ta + o;
-  float* tc = tb + o;
-  float* dm = tc + o;
-  // U pairs (U[i][al], U[i][al]), 16-byte aligned for 128-bit loads
-  const int uoff = (2 * blk + 3 * o2p + 4 * o + 3) & ~3;
-  float* U2 = reinterpret_cast<float*>(smraw) + uoff;
-  // (pa|qb) etc. from the FP32 copy ovT[x][y][p][q] = (px|qy): o^2 consecutive floats per slice
-  const float* oab = ovT + (1LL * a * v + b) * o2;
-  const float* oac = ovT + (1LL * a * v + c) * o2;
-  const float* obc = ovT + (1LL * b * v + c) * o2;
-  for (int idx = threadIdx.x; idx < o2; idx += blockDim.x) {
-    const int p = idx / o, q = idx % o;
-    Sab[p * P1 + q] = oab[idx];
-    Sac[p * P1 + q] = oac[idx];
-    Sbc[p * P1 + q] = obc[idx];
-  }
-  for (int y = threadIdx.x; y < o; y += blockDim.x) {
-    const double ex3 = (eps[o + a] + eps[o + b] + eps[o + c]) / 3.0;  // FP64 in these o threads only
-    ta[y] = static_cast<float>(t1[y * v + a]);
-    tb[y] = static_cast<float>(t1[y * v + b]);
-    tc[y] = static_cast<float>(t1[y * v + c]);
-    dm[y] = static_cast<float>(ex3 - eps[y]);
-  }
-  for (int idx = threadIdx.x; idx < o * NLO; idx += blockDim.x) {
-    const float u = static_cast<float>(U[idx]);
-    U2[2 * idx] = u;
-    U2[2 * idx + 1] = u;
-  }
-  __syncthreads();
-  const float* Wb = W + slot * slot_stride + static_cast<long long>(a) * o3;
-  // W is stored [i][k][j] (j fastest). Each thread owns pairs (j, k) = (y1, y2) (consecutive threads:
-  // consecutive j, so every load instruction reads a contiguous row of W) and walks i = y0 with eight
-  // loads in flight; the terms that depend on (j, k) only (t1 of b and c, (bj|ck), d_j + d_k) stay in
-  // registers across the walk.
-  constexpr int kLoads = 8;
-  for (int jk = threadIdx.x; jk < o2; jk += blockDim.x) {
-    const int y1 = jk % o, y2 = jk / o;
-    const float tcv = tc[y2], tbv = tb[y1], sbc = Sbc[y1 * P1 + y2], d12 = dm[y1] + dm[y2];
-    const float* wp = Wb + jk;
-    float2* dst = swv + y1 * S1 + y2;
-    for (int i0 = 0; i0 < o; i0 += kLoads) {
-      float wr[kLoads];
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u) wr[u] = i0 + u < o ? wp[static_cast<long long>(i0 + u) * o2] : 0.f;
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u) {
-        const int y0 = i0 + u;
-        if (y0 < o) {
-          const float disc = Sab[y0 * P1 + y1] * tcv + Sac[y0 * P1 + y2] * tbv + sbc * ta[y0];
-          const float sc = rsqrtf(dm[y0] + d12);
-          dst[y0 * S0] = make_float2(wr[u] * sc, (wr[u] + disc) * sc);
-        }
+// Unordered occupied triples, i | j << 8 | k << 16 (nocc <= 255), grouped by the gaps between their members
+// around the circle 0 .. o-1: consecutive entries are one triple shifted by one orbital, so that consecutive
+// threads read the staged block at a constant odd stride whatever the placement (lexicographic order cost four
+// bank conflicts per load). Gap sequences (g1, g2, o - g1 - g2), one per class of cyclic rotations; one warp.
+__global__ void k_tri_table(int o, unsigned* __restrict__ tri) {
+  int pos = 0;
+  for (int g1 = 0; g1 <= o / 3; ++g1) {
+    for (int g2 = g1; g2 <= o - 2 * g1; ++g2) {
+      const int g3 = o - g1 - g2;
+      // the smallest rotation stands for the class: g1 <= g2, g1 <= g3, and with g3 = g1 only g2 = g1
+      if (g3 == g1 && g2 != g1) continue;
+      const int n = g1 == g2 && g2 == g3 ? g1 : o;  // equal gaps: the triple repeats after a third of the circle
+      for (int i = threadIdx.x; i < n; i += 32) {
+        const int j = (i + g1) % o, k = (i + g1 + g2) % o;
+        tri[pos + i] = static_cast<unsigned>(i) | static_cast<unsigned>(j) << 8 | static_cast<unsigned>(k) << 16;
       }
+      pos += n;
     }
   }
-  __syncthreads();
-  // placements and orderings as in k_t_energy_staged
-  constexpr int PM[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-  const int x0 = a, x1 = b, x2 = c;
-  auto X = [&](int p) { return p == 0 ? x0 : (p == 1 ? x1 : x2); };
-  auto SS = [&](int p) { return p == 0 ? S0 : (p == 1 ? S1 : 1); };
-  const bool distinct = a < b && b < c;
-  bool act[6];
-#pragma unroll
-  for (int pi = 0; pi < 6; ++pi) {
-    bool dup = false;
-    if (!distinct) {
-#pragma unroll
-      for (int q = 0; q < pi; ++q)
-        dup = dup || (X(PM[q][0]) == X(PM[pi][0]) && X(PM[q][1]) == X(PM[pi][1]) && X(PM[q][2]) == X(PM[pi][2]));
-    }
-    act[pi] = !dup;
-  }
-  constexpr int NL = NLO > 0 ? NLO : 1;
-  // FP32 sums run over one (j, k) only; partials across (j, k) in compensated FP32 (CSum)
-  CSum r_can{0.f, 0.f}, r_frag{0.f, 0.f};
-  for (int jk = threadIdx.x; jk < o2; jk += blockDim.x) {
-    const int j = jk / o, k = jk % o;
-    int off[6], si[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      off[q] = j * SS(PM[q][1]) + k * SS(PM[q][2]);
-      si[q] = SS(PM[q][0]);
-    }
-    float acc = 0.f;
-    if (distinct) {
-      // a < b < c: all six orderings are distinct. With w_q, v_q the six placements (q = 0, 3, 4 the
-      // cyclic ones, 1, 2, 5 the others), ordering q has z_q = 3 w_q + S (S the sum of w over q's class)
-      // and y_q = v_q - v_r with r = rev(q) the placement of the reversed slots (0<->5, 3<->1, 4<->2,
-      // always of the other class), so y_r = -y_q. Each pair then contributes
-      // (z_q - z_r) y_q = (3 (w_q - w_r) + S_cyc - S_oth) y_q to the canonical sum, and, since the
-      // i-sums of y_r are minus those of y_q, (sum_i U (z_q - z_r)) (sum_i U y_q) to the projected one:
-      // three products per (i, j, k) instead of six, the same quantities.
-      float2 zp[3][NL];  // (sum_i U (z_q - z_r), sum_i U y_q) per pair and LO
-#pragma unroll
-      for (int h = 0; h < 3; ++h)
-#pragma unroll
-        for (int al = 0; al < NL; ++al) zp[h][al] = make_float2(0.f, 0.f);
-#pragma unroll (OC > 0 ? OC : 2)
-      for (int i = 0; i < o; ++i) {
-        float2 p[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-          p[q] = swv[off[q]];
-          off[q] += si[q];
-        }
-        const float dS = (p[0].x + p[3].x + p[4].x) - (p[1].x + p[2].x + p[5].x);
-        const float2 d0 = make_float2(fmaf(3.f, p[0].x - p[5].x, dS), p[0].y - p[5].y);
-        const float2 d1 = make_float2(fmaf(3.f, p[3].x - p[1].x, dS), p[3].y - p[1].y);
-        const float2 d2 = make_float2(fmaf(3.f, p[4].x - p[2].x, dS), p[4].y - p[2].y);
-        acc = fmaf(d0.x, d0.y, acc);
-        acc = fmaf(d1.x, d1.y, acc);
-        acc = fmaf(d2.x, d2.y, acc);
-        if constexpr (NLO > 0) {
-          float2 u2[NL];
-          if constexpr (NLO == 1) {
-            u2[0] = reinterpret_cast<const float2*>(U2)[i];
-          } else {
-#pragma unroll
-            for (int h = 0; h < NLO / 2; ++h) {
-              const float4 t = reinterpret_cast<const float4*>(U2)[i * (NLO / 2) + h];
-              u2[2 * h] = make_float2(t.x, t.y);
-              u2[2 * h + 1] = make_float2(t.z, t.w);
-            }
-          }
-#pragma unroll
-          for (int al = 0; al < NLO; ++al) {
-            zp[0][al] = __ffma2_rn(u2[al], d0, zp[0][al]);
-            zp[1][al] = __ffma2_rn(u2[al], d1, zp[1][al]);
-            zp[2][al] = __ffma2_rn(u2[al], d2, zp[2][al]);
-          }
-        }
-      }
-      csum_add(r_can, acc);
-      float f = 0.f;
-#pragma unroll
-      for (int h = 0; h < 3; ++h)
-#pragma unroll
-        for (int al = 0; al < NLO; ++al) f += zp[h][al].x * zp[h][al].y;
-      csum_add(r_frag, f);
-      continue;
-    }
-    float2 zy[6][NL];  // (sum_i U z, sum_i U y) per ordering and LO
-#pragma unroll
-    for (int pi = 0; pi < 6; ++pi)
-#pragma unroll
-      for (int al = 0; al < NL; ++al) zy[pi][al] = make_float2(0.f, 0.f);
-    for (int i = 0; i < o; ++i) {
-      float2 p[6];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        p[q] = swv[off[q]];
-        off[q] += si[q];
-      }
-      float2 u2[NL];
-      if constexpr (NLO == 1) {
-        u2[0] = reinterpret_cast<const float2*>(U2)[i];
-      } else if constexpr (NLO > 1) {
-#pragma unroll
-        for (int h = 0; h < NLO / 2; ++h) {
-          const float4 t = reinterpret_cast<const float4*>(U2)[i * (NLO / 2) + h];
-          u2[2 * h] = make_float2(t.x, t.y);
-          u2[2 * h + 1] = make_float2(t.z, t.w);
-        }
-      }
-#pragma unroll
-      for (int pi = 0; pi < 6; ++pi) {
-        if (!act[pi]) continue;
-        const int p0 = PM[pi][0], p1 = PM[pi][1], p2 = PM[pi][2];
-        auto idx = [&](int s0, int s1) {
-          return s0 == 0 ? (s1 == 1 ? 0 : 1) : (s0 == 1 ? (s1 == 0 ? 2 : 3) : (s1 == 0 ? 4 : 5));
-        };
-        const float z = 4 * p[idx(p0, p1)].x + p[idx(p1, p2)].x + p[idx(p2, p0)].x;
-        const float y = p[idx(p0, p1)].y - p[idx(p2, p1)].y;
-        acc += z * y;
-        const float2 zyv = make_float2(z, y);
-#pragma unroll
-        for (int al = 0; al < NLO; ++al) zy[pi][al] = __ffma2_rn(u2[al], zyv, zy[pi][al]);
-      }
-    }
-    csum_add(r_can, acc);
-    float f = 0.f;
-#pragma unroll
-    for (int pi = 0; pi < 6; ++pi)
-#pragma unroll
-      for (int al = 0; al < NLO; ++al) f += zy[pi][al].x * zy[pi][al].y;
-    csum_add(r_frag, f);
-  }
-  csum_block_out(r_can, r_frag, out, blk_id);
-}
-
-// Block energy of the mixed path when only w fits in shared memory (nocc 29..35 at 200 KB): w = W s is
-// staged, v = w + disc s is formed where it is read. s depends on the unordered triple (i, j, k), so one
-// rsqrt per (i, j, k) serves all six placements; of the fifteen slice / t1 values the six placements'
-// disconnected terms need at fixed (j, k), the ones that do not involve i stay in registers across the
-// i walk. Orderings are paired as in k_t_energy_f32 when a < b < c. 512 threads per block (two (j, k)
-// pairs per thread at nocc 32) with NLO <= 2, 256 above.
-template <int NLO>
-__global__ void __launch_bounds__(NLO <= 2 ? 512 : 256, 1)
-    k_t_energy_vfly(const float* __restrict__ W, long long slot_stride, int b, int c0, int o, int v,
-                    const double* __restrict__ eps, const double* __restrict__ t1, const float* __restrict__ ovT,
-                    const double* __restrict__ U, double* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int slot = blockIdx.y, a = blockIdx.x;
-  const int c = c0 + slot;
-  const long long blk_id = static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x;
-  const int o2 = o * o, o3 = o2 * o;
-  const int S1 = o + 1, S0 = o * S1 + 1;
-  const int blk = o * S0;
-  float* sw = reinterpret_cast<float*>(smraw);  // w at y0 * S0 + y1 * S1 + y2
-  float* fs = sw + blk;
-  const int P1 = o + 1, o2p = o * P1;
-  float* Sab = fs;  // (y0 a|y1 b)
-  float* Sac = Sab + o2p;
-  float* Sbc = Sac + o2p;
-  float* ta = Sbc + o2p;
-  float* tb = ta + o;
-  float* tc = tb + o;
-  float* dm = tc + o;
-  const int uoff = (blk + 3 * o2p + 4 * o + 3) & ~3;
-  float* U2 = sw + uoff;  // (U[i][al], U[i][al]) pairs
-  const float* oab = ovT + (1LL * a * v + b) * o2;
-  const float* oac = ovT + (1LL * a * v + c) * o2;
-  const float* obc = ovT + (1LL * b * v + c) * o2;
-  for (int idx = threadIdx.x; idx < o2; idx += blockDim.x) {
-    const int p = idx / o, q = idx % o;
-    Sab[p * P1 + q] = oab[idx];
-    Sac[p * P1 + q] = oac[idx];
-    Sbc[p * P1 + q] = obc[idx];
-  }
-  for (int y = threadIdx.x; y < o; y += blockDim.x) {
-    const double ex3 = (eps[o + a] + eps[o + b] + eps[o + c]) / 3.0;  // FP64 in these o threads only
-    ta[y] = static_cast<float>(t1[y * v + a]);
-    tb[y] = static_cast<float>(t1[y * v + b]);
-    tc[y] = static_cast<float>(t1[y * v + c]);
-    dm[y] = static_cast<float>(ex3 - eps[y]);
-  }
-  for (int idx = threadIdx.x; idx < o * NLO; idx += blockDim.x) {
-    const float u = static_cast<float>(U[idx]);
-    U2[2 * idx] = u;
-    U2[2 * idx + 1] = u;
-  }
-  __syncthreads();
-  const float* Wb = W + slot * slot_stride + static_cast<long long>(a) * o3;
-  // staging: thread-owned (j, k) pairs walking i, as in k_t_energy_f32 (w only)
-  constexpr int kLoads = 8;
-  for (int jk = threadIdx.x; jk < o2; jk += blockDim.x) {
-    const int y1 = jk % o, y2 = jk / o;
-    const float d12 = dm[y1] + dm[y2];
-    const float* wp = Wb + jk;
-    float* dst = sw + y1 * S1 + y2;
-    for (int i0 = 0; i0 < o; i0 += kLoads) {
-      float wr[kLoads];
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u) wr[u] = i0 + u < o ? wp[static_cast<long long>(i0 + u) * o2] : 0.f;
-#pragma unroll
-      for (int u = 0; u < kLoads; ++u)
-        if (i0 + u < o) dst[(i0 + u) * S0] = wr[u] * rsqrtf(dm[i0 + u] + d12);
-    }
-  }
-  __syncthreads();
-  constexpr int PM[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-  const int x0 = a, x1 = b, x2 = c;
-  auto X = [&](int p) { return p == 0 ? x0 : (p == 1 ? x1 : x2); };
-  auto SS = [&](int p) { return p == 0 ? S0 : (p == 1 ? S1 : 1); };
-  const bool distinct = a < b && b < c;
-  bool act[6];
-#pragma unroll
-  for (int pi = 0; pi < 6; ++pi) {
-    bool dup = false;
-    if (!distinct) {
-#pragma unroll
-      for (int q = 0; q < pi; ++q)
-        dup = dup || (X(PM[q][0]) == X(PM[pi][0]) && X(PM[q][1]) == X(PM[pi][1]) && X(PM[q][2]) == X(PM[pi][2]));
-    }
-    act[pi] = !dup;
-  }
-  constexpr int NL = NLO > 0 ? NLO : 1;
-  // FP32 sums over one (j, k); partials across (j, k) in compensated FP32 (CSum)
-  CSum r_can{0.f, 0.f}, r_frag{0.f, 0.f};
-  for (int jk = threadIdx.x; jk < o2; jk += blockDim.x) {
-    const int j = jk / o, k = jk % o;
-    int off[6], si[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      off[q] = j * SS(PM[q][1]) + k * SS(PM[q][2]);
-      si[q] = SS(PM[q][0]);
-    }
-    // (j, k)-only factors of the disconnected terms d(y0,y1,y2) = Sab[y0][y1] tc[y2] + Sac[y0][y2] tb[y1]
-    // + Sbc[y1][y2] ta[y0] of the placements (i,j,k), (i,k,j), (j,i,k), (k,i,j), (j,k,i), (k,j,i)
-    const float sbc_jk = Sbc[j * P1 + k], sbc_kj = Sbc[k * P1 + j], sac_jk = Sac[j * P1 + k],
-                sac_kj = Sac[k * P1 + j], sab_jk = Sab[j * P1 + k], sab_kj = Sab[k * P1 + j];
-    const float taj = ta[j], tak = ta[k], tbj = tb[j], tbk = tb[k], tcj = tc[j], tck = tc[k];
-    const float djk = dm[j] + dm[k];
-    float acc = 0.f;
-    float2 zy[6][NL];
-#pragma unroll
-    for (int h = 0; h < 6; ++h)
-#pragma unroll
-      for (int al = 0; al < NL; ++al) zy[h][al] = make_float2(0.f, 0.f);
-    for (int i = 0; i < o; ++i) {
-      float w[6], vv[6];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        w[q] = sw[off[q]];
-        off[q] += si[q];
-      }
-      const float s = rsqrtf(dm[i] + djk);
-      const float sab_ij = Sab[i * P1 + j], sab_ji = Sab[j * P1 + i], sab_ik = Sab[i * P1 + k],
-                  sab_ki = Sab[k * P1 + i];
-      const float sac_ij = Sac[i * P1 + j], sac_ji = Sac[j * P1 + i], sac_ik = Sac[i * P1 + k],
-                  sac_ki = Sac[k * P1 + i];
-      const float sbc_ij = Sbc[i * P1 + j], sbc_ji = Sbc[j * P1 + i], sbc_ik = Sbc[i * P1 + k],
-                  sbc_ki = Sbc[k * P1 + i];
-      const float tai = ta[i], tbi = tb[i], tci = tc[i];
-      vv[0] = w[0] + (sab_ij * tck + sac_ik * tbj + sbc_jk * tai) * s;  // (i, j, k)
-      vv[1] = w[1] + (sab_ik * tcj + sac_ij * tbk + sbc_kj * tai) * s;  // (i, k, j)
-      vv[2] = w[2] + (sab_ji * tck + sac_jk * tbi + sbc_ik * taj) * s;  // (j, i, k)
-      vv[3] = w[3] + (sab_ki * tcj + sac_kj * tbi + sbc_ij * tak) * s;  // (k, i, j)
-      vv[4] = w[4] + (sab_jk * tci + sac_ji * tbk + sbc_ki * taj) * s;  // (j, k, i)
-      vv[5] = w[5] + (sab_kj * tci + sac_ki * tbj + sbc_ji * tak) * s;  // (k, j, i)
-      float2 u2[NL];
-      if constexpr (NLO == 1) {
-        u2[0] = reinterpret_cast<const float2*>(U2)[i];
-      } else if constexpr (NLO > 1) {
-#pragma unroll
-        for (int h = 0; h < NLO / 2; ++h) {
-          const float4 t = reinterpret_cast<const float4*>(U2)[i * (NLO / 2) + h];
-          u2[2 * h] = make_float2(t.x, t.y);
-          u2[2 * h + 1] = make_float2(t.z, t.w);
-        }
-      }
-      if (distinct) {
-        // pairs (0, 5), (3, 1), (4, 2): (z_q - z_r, y_q), see k_t_energy_f32
-        const float dS = (w[0] + w[3] + w[4]) - (w[1] + w[2] + w[5]);
-        const float2 d0 = make_float2(fmaf(3.f, w[0] - w[5], dS), vv[0] - vv[5]);
-        const float2 d1 = make_float2(fmaf(3.f, w[3] - w[1], dS), vv[3] - vv[1]);
-        const float2 d2 = make_float2(fmaf(3.f, w[4] - w[2], dS), vv[4] - vv[2]);
-        acc = fmaf(d0.x, d0.y, acc);
-        acc = fmaf(d1.x, d1.y, acc);
-        acc = fmaf(d2.x, d2.y, acc);
-#pragma unroll
-        for (int al = 0; al < NLO; ++al) {
-          zy[0][al] = __ffma2_rn(u2[al], d0, zy[0][al]);
-          zy[1][al] = __ffma2_rn(u2[al], d1, zy[1][al]);
-          zy[2][al] = __ffma2_rn(u2[al], d2, zy[2][al]);
-        }
-      } else {
-#pragma unroll
-        for (int pi = 0; pi < 6; ++pi) {
-          if (!act[pi]) continue;
-          const int p0 = PM[pi][0], p1 = PM[pi][1], p2 = PM[pi][2];
-          auto idx = [&](int s0, int s1) {
-            return s0 == 0 ? (s1 == 1 ? 0 : 1) : (s0 == 1 ? (s1 == 0 ? 2 : 3) : (s1 == 0 ? 4 : 5));
-          };
-          const float z = 4 * w[idx(p0, p1)] + w[idx(p1, p2)] + w[idx(p2, p0)];
-          const float y = vv[idx(p0, p1)] - vv[idx(p2, p1)];
-          acc += z * y;
-          const float2 zyv = make_float2(z, y);
-#pragma unroll
-          for (int al = 0; al < NLO; ++al) zy[pi][al] = __ffma2_rn(u2[al], zyv, zy[pi][al]);
-        }
-      }
-    }
-    csum_add(r_can, acc);
-    float f = 0.f;
-#pragma unroll
-    for (int pi = 0; pi < 6; ++pi)
-#pragma unroll
-      for (int al = 0; al < NLO; ++al) f += zy[pi][al].x * zy[pi][al].y;
-    csum_add(r_frag, f);
-  }
-  csum_block_out(r_can, r_frag, out, blk_id);
 }
 
 // Per-c tables of the batched (T) terms, one entry per (b, c >= b) in b-major order (the order of the
@@ -922,6 +490,7 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
   p.tpart = static_cast<size_t>(p.nblk + 256) * 2 * 8;  // block partials, then 256 first-pass sums
   p.batch = sizeof(BatchEntry) * static_cast<size_t>(std::max(1LL, vv / 2 + v));  // one entry per (b, c >= b)
   p.u = static_cast<size_t>(o) * 8 * 8;  // U padded to at most 8 LOs
+  p.tri = static_cast<size_t>(tri_count(std::min(o, kMaxStagedOcc))) * 4;  // unordered occupied triples
   p.ovt = bf ? static_cast<size_t>(vv * oo) * 4 : 0;  // FP32 (ia|jb) in block-energy order (mixed)
   auto al = [](size_t x) { return (std::max<size_t>(x, 256) + 255) / 256 * 256; };
   // FP64: the digit planes of the four operands, cut once per call instead of in every product that reads
@@ -935,7 +504,7 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
     p.total += 2 * al(p.slxt) + 2 * al(p.slto);
   }
   p.total += 2 * al(p.xt) + 2 * al(p.to) + al(p.ovoo) + al(p.pbvv) + al(p.ovvv_chunk) + al(p.w) + al(p.tpart) +
-            2 * al(p.batch) + al(p.u) + (bf ? al(p.ovt) : 0);
+            2 * al(p.batch) + al(p.u) + (bf ? al(p.ovt) + al(p.tri) : 0);
   return p;
 }
 
@@ -1128,16 +697,17 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   count_launch();
   k_batch_tables<<<(v + 127) / 128, 128, 0, s>>>(o, v, welems, dbat, dbat12);
 
-  const long long sblk = 1LL * o * (1LL * o * (o + 1) + 1);  // padded w / v block of the energy kernel
-  // slices, t1 columns, d_m and U (up to 8 LOs, duplicated into pairs, plus 16-byte alignment)
+  // Block energy kernel. Mixed: w and v staged side by side while they fit (nocc <= 28: 182 KB at 28), one
+  // value per element up to nocc 37 (203 KB), at most 8 LOs; FP64: w and v or w alone within 200 KB.
+  // Otherwise the generic kernel (any nocc and nlo, nothing staged).
+  const long long sblk = 1LL * o * (1LL * o * (o + 1) + 1);  // padded w / v block of the FP64 kernel
   const long long small_smem = (3LL * o * (o + 1) + 4LL * o + 16LL * o + 4) * wsz;
   const bool staged_full = 2LL * sblk * wsz + small_smem <= 200LL * 1024;
-  const bool staged = (staged_full || sblk * wsz + small_smem <= 200LL * 1024) && nlo <= 8;
-  // (the staged kernel reads U padded to its compile-time LO count)
-  const size_t esmem = (staged_full ? 2 : 1) * sblk * wsz + static_cast<size_t>(small_smem);
-  // the energy kernel is compiled for 0, 1, 2, 4 or 8 LOs; U is zero-padded to the next size
-  // (the generic kernel, used when the staged ones are not, reads U as given: any nlo)
-  const int nlo_t = nlo == 0 ? 0 : nlo <= 1 ? 1 : nlo <= 2 ? 2 : nlo <= 4 ? 4 : 8;
+  const bool staged =
+      (bf ? o <= kMaxStagedOcc : staged_full || sblk * wsz + small_smem <= 200LL * 1024) && nlo <= 8;
+  // the FP64 kernel is compiled for 0, 1, 2, 4 or 8 LOs: U zero-padded to the next size
+  const int nlo_t = bf || nlo == 0 ? nlo : nlo <= 1 ? 1 : nlo <= 2 ? 2 : nlo <= 4 ? 4 : 8;
+  const size_t esmem = (staged_full ? 2 : 1) * sblk * wsz + static_cast<size_t>(small_smem);  // FP64 kernel
   double* dUp = nullptr;
   if (staged && nlo_t > 0) {
     dUp = static_cast<double*>(tmp_alloc(tp.u));
@@ -1149,34 +719,28 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     cudaMemsetAsync(dUp, 0, static_cast<size_t>(o) * nlo_t * 8, s);
     cudaMemcpy2DAsync(dUp, nlo_t * 8, U, nlo * 8, nlo * 8, o, cudaMemcpyDeviceToDevice, s);
   }
-  float* ovT = nullptr;  // k_t_energy_f32 / k_t_energy_vfly read (ia|jb) from this FP32 copy
+  float* ovT = nullptr;  // the FP32 kernels read (ia|jb) from this copy
+  unsigned* tri = nullptr;
   if (bf && staged) {
     ovT = static_cast<float*>(tmp_alloc(tp.ovt));
-    if (!ovT) {
+    tri = static_cast<unsigned*>(tmp_alloc(tp.tri));
+    if (!ovT || !tri) {
       cleanup();
       set_error("lnocc_triples: device allocation failed (ovT)");
       return LNOCC_ENOMEM;
     }
-    count_launch();
+    count_launch(2);
     k_ovov_t<<<1216, 256, 0, s>>>(ovov, ovT, o, v);
+k_tri_table<<<1, 32, 0, s>>>(o, tri);
   }
   auto energy_launch = [&](const void* Wp, long long Sc, int b, int c0, int na, int nc, double* part) {
+    if (bf) {
+      launch_block_energy(EnergyArgs{static_cast<const float*>(Wp), Sc, b, c0, o, v, eps, t1, ovT, dUp, nlo, tri, part, na, nc},
+                          s);
+      return;
+    }
     dim3 grid(na, nc);
     count_launch();
-    // FP32 W with w and v staged: k_t_energy_f32; otherwise the generic staged kernel
-#define LN_F(K)                                                                                          \
-  do {                                                                                                   \
-    if (staged_full)                                                                                     \
-      if (o == 16)                                                                                       \
-        k_t_energy_f32<K, 16><<<grid, 256, esmem, s>>>(static_cast<const float*>(Wp), Sc, b, c0, o, v, eps, \
-                                                       t1, ovT, dUp, part);                              \
-      else                                                                                               \
-        k_t_energy_f32<K, 0><<<grid, 256, esmem, s>>>(static_cast<const float*>(Wp), Sc, b, c0, o, v, eps,  \
-                                                      t1, ovT, dUp, part);                               \
-    else                                                                                                 \
-      k_t_energy_vfly<K><<<grid, K <= 2 ? 512 : 256, esmem, s>>>(static_cast<const float*>(Wp), Sc, b, c0, o, \
-                                                                 v, eps, t1, ovT, dUp, part);            \
-  } while (0)
 #define LN_D(K)                                                                                          \
   do {                                                                                                   \
     if (staged_full)                                                                                     \
@@ -1188,60 +752,34 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
                                                                           b, c0, o, v, eps, t1, ovov, dUp, \
                                                                           nlo_t, part);                  \
   } while (0)
-    if (bf) {
-      switch (nlo_t) {
-        case 0: LN_F(0); break;
-        case 1: LN_F(1); break;
-        case 2: LN_F(2); break;
-        case 4: LN_F(4); break;
-        default: LN_F(8); break;
-      }
-    } else {
-      switch (nlo_t) {
-        case 0: LN_D(0); break;
-        case 1: LN_D(1); break;
-        case 2: LN_D(2); break;
-        case 4: LN_D(4); break;
-        default: LN_D(8); break;
-      }
+    switch (nlo_t) {
+      case 0: LN_D(0); break;
+      case 1: LN_D(1); break;
+      case 2: LN_D(2); break;
+      case 4: LN_D(4); break;
+      default: LN_D(8); break;
     }
-#undef LN_F
 #undef LN_D
   };
-  if (staged) {
-    // The attribute is per kernel and process-wide: set it once to the largest size the staged
-    // kernel is ever launched with (the 200 KB cap above), so that concurrent calls on fragments of
-    // other sizes never lower it under one another's launches.
+  if (staged && !bf) {
+    // The attribute is per kernel and process-wide: set it once to the largest size a staged kernel can be
+    // launched with, so that concurrent calls on fragments of other sizes never lower it under one
+    // another's launches.
     static std::once_flag once;
     std::call_once(once, [] {
-      auto attr = [](const void* fn) {
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      auto attr = [](const void* fn, int bytes) {
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       };
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<0, 0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<0, 16>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<1, 0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<1, 16>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<2, 0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<2, 16>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<4, 0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<4, 16>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<8, 0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_f32<8, 16>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 0, false>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 1, false>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 2, false>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 4, false>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 8, false>));
-      attr(reinterpret_cast<const void*>(k_t_energy_vfly<0>));
-      attr(reinterpret_cast<const void*>(k_t_energy_vfly<1>));
-      attr(reinterpret_cast<const void*>(k_t_energy_vfly<2>));
-      attr(reinterpret_cast<const void*>(k_t_energy_vfly<4>));
-      attr(reinterpret_cast<const void*>(k_t_energy_vfly<8>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 0, true>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 1, true>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 2, true>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 4, true>));
-      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 8, true>));
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 0, false>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 1, false>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 2, false>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 4, false>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 8, false>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 0, true>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 1, true>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 2, true>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 4, true>), 200 * 1024);
+      attr(reinterpret_cast<const void*>(k_t_energy_staged<double, double, 8, true>), 200 * 1024);
     });
   }
   auto omap = [&](double beta) {
