@@ -54,11 +54,10 @@ extern "C" {
 
 /* (T) contraction launches on the mixed path. PER_TERM: one launch per W term (sigma1 + sigma2, sigma3,
  * sigma4, sigma6, sigma5) per chunk. GROUPED: two launches per chunk; the first runs sigma1 + sigma2,
- * sigma3 and sigma5 of one (c, 128-row tile of (a, x)) block back to back in one CTA (the block stays
- * in L2 between its store and its two reductions), the second sigma4 and sigma6. GROUPED needs
- * nocc = 16 or 32 (128 rows hold whole a values; the (y, z) plane is one or four 256-column
- * accumulator tiles); AUTO takes it there and PER_TERM elsewhere, and GROUPED falls back to PER_TERM
- * for other nocc. */
+ * sigma3 and sigma5 of one (c, row tile of (a, x)) block back to back in one CTA (the block stays in L2
+ * between its store and its two reductions), the second sigma4 and sigma6. GROUPED needs nocc from 4 to
+ * 32 (a row tile holds whole a values); AUTO takes it there and PER_TERM elsewhere, and GROUPED falls back
+ * to PER_TERM for other nocc. */
 #define LNOCC_TK_AUTO 0
 #define LNOCC_TK_PER_TERM 1
 #define LNOCC_TK_GROUPED 2

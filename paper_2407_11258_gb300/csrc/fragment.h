@@ -33,7 +33,7 @@ struct Consts {
 struct TriplesPlan {
   size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, tri, slxt, slto, total;
   long long welems, nblk;
-  int bc;
+  int bc, jp;
 };
 TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb);
 // Elements (FP64-sized) of each of the two packing scratch buffers of a fragment (ccsd.cu).

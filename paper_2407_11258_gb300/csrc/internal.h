@@ -128,6 +128,22 @@ struct GrpSpec {
 void gemm_grouped(const Packed* const ops[4], const int box_rows[4], const GrpSpec& g, const OutMap* Cg, int ncg,
                   cudaStream_t s, int* dstatus);
 
+// A grouped (T) launch for any nocc from 4 to 32 (triples_gemm.cu). The caller sets kind, b, c0, nc, o, bvo, vo
+// and Sc; the rest is derived.
+struct TgSpec {
+  int kind;         // 1: sigma1 + sigma2, sigma3, sigma5; 2: sigma4, sigma6
+  int b, c0, nc;    // slab b, the chunk's first c and its number of c
+  int o, bvo, vo;   // nocc, b nvir nocc, nvir nocc
+  long long Sc;     // W elements per c
+  int oo, jp;       // nocc^2; nocc rounded up to 4 (row length of W)
+  int ta;           // units (a, or (a, i) pairs) of a 128-row tile
+  int mt, nreg;     // row tiles per c or block of c; regions
+  int ncol, nk;     // column tiles of a plane (kind 1); outer column values of a tile
+  int nkb;          // K blocks of 32 per term
+};
+// ops: kind 1 XT1, TO, XT2, TOT; kind 2 TO, XT2, XT2, XT1 (BF16 hi/lo, K columns used).
+void gemm_grouped_any(const Packed* const ops[4], TgSpec g, float* W, int K, cudaStream_t s, int* dstatus);
+
 // Workspaces of the contraction engine, provided by its caller: split-K partials (p, cap FP64 elements)
 // and the digit planes of FP64 products (sl, sl_bytes). Per host thread: each thread drives its own
 // fragment and stream.

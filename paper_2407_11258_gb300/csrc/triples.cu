@@ -53,17 +53,17 @@ template <typename TW>
 __global__ void k_t_energy(const TW* __restrict__ W, long long slot_stride, int b, int c0, int o, int v,
                            const double* __restrict__ eps, const double* __restrict__ t1,
                            const double* __restrict__ ovov, const double* __restrict__ U, int nlo,
-                           double* __restrict__ out) {
+                           double* __restrict__ out, int jp) {
   const int slot = blockIdx.y;
   const int a = blockIdx.x;
   const int c = c0 + slot;
-  const long long oblk = 1LL * o * o * o;
+  const long long oblk = 1LL * o * o * jp;
   const long long blk_id = static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x;
   const TW* Wb = W + slot * slot_stride + a * oblk;
   const int x[3] = {a, b, c};
   const double ex = eps[o + a] + eps[o + b] + eps[o + c];
   const long long ov = 1LL * o * v;
-  auto widx = [&](int y0, int y1, int y2) { return (1LL * y0 * o + y2) * o + y1; };  // W stored [a][i][k][j]
+  auto widx = [&](int y0, int y1, int y2) { return (1LL * y0 * o + y2) * jp + y1; };  // W stored [a][i][k][j], rows of jp
   // w and v of the block at occupied (y0, y1, y2)
   auto wv = [&](int y0, int y1, int y2, double& w, double& vv) {
     const double Wv = static_cast<double>(Wb[widx(y0, y1, y2)]);
@@ -347,14 +347,14 @@ __global__ void k_tri_table(int o, unsigned* __restrict__ tri) {
 
 // Per-c tables of the batched (T) terms, one entry per (b, c >= b) in b-major order (the order of the
 // chunk plan: entry (b, c) at b v - b (b - 1) / 2 + c - b). For W chunks of ncmax(b) = max(1, welems /
-// ((b + 1) o^3)) values of c, c sits at position q = (c - b) mod ncmax(b) of its chunk. bat: sigma5
+// ((b + 1) o^2 jp)) values of c, c sits at position q = (c - b) mod ncmax(b) of its chunk. bat: sigma5
 // (rows (c, a, k) of XT2 against rows (b, i, j) of TOT); bat12: sigma1 (rows (b, a, i) of XT1 against rows
 // (c, k, j) of TO) then sigma2 (rows (c, a, i) of XT1 against rows (b, k, j) of TOT) into one accumulator.
-__global__ void k_batch_tables(int o, int v, long long welems, BatchEntry* __restrict__ bat,
+__global__ void k_batch_tables(int o, int v, int jp, long long welems, BatchEntry* __restrict__ bat,
                                BatchEntry* __restrict__ bat12) {
-  const long long oo = 1LL * o * o, ooo = oo * o;
+  const long long oo = 1LL * o * o, ooj = oo * jp;
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < v; b += gridDim.x * blockDim.x) {
-    const long long slab = 1LL * (b + 1) * ooo;
+    const long long slab = (b + 1) * ooj;
     const long long ncmax = welems / slab > 1 ? welems / slab : 1;
     const long long base = 1LL * b * v - 1LL * b * (b - 1) / 2;
     const int Ma = (b + 1) * o;
@@ -480,10 +480,12 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
   p.ovvv_chunk = static_cast<size_t>(p.bc) * o * vv * 8;
   // W chunk: up to chunk_mb (fewer, larger contraction launches measured faster than chunks that fit
   // L2), but never more than the largest slab (b + 1)(v - b) o^3 needs, and at least one c of a slab
+  p.jp = bf ? round_up(o, 4) : o;  // row length of W: 16-byte rows for the copies of the mixed path
+  const long long ooj = oo * p.jp;
   long long max_slab = 0;
-  for (int bb = 0; bb < v; ++bb) max_slab = std::max(max_slab, 1LL * (bb + 1) * (v - bb) * ooo);
+  for (int bb = 0; bb < v; ++bb) max_slab = std::max(max_slab, 1LL * (bb + 1) * (v - bb) * ooj);
   const long long cmb = chunk_mb > 0 ? chunk_mb : 768;
-  p.welems = std::max<long long>(std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab), v * ooo);
+  p.welems = std::max<long long>(std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab), v * ooj);
   p.w = static_cast<size_t>(p.welems) * esz;
   p.nblk = 0;
   for (int b = 0; b < v; ++b) p.nblk += 1LL * (b + 1) * (v - b);
@@ -658,6 +660,8 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
 
   // ---- slabs of fixed b: virtual c in [b, v) in chunks, a in [0, b]; W_chunk[c - c0][a][i][j][k]
   const size_t wsz = bf ? 4 : 8;
+  const int jp = tp.jp;
+  const long long ooj = oo * jp;  // W elements of one (c, a)
   const long long welems = tp.welems;
   void* W = tmp_alloc(tp.w);
   const long long nblk_total = tp.nblk;
@@ -672,7 +676,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   {
     long long part = 0;
     for (int b = 0; b < v; ++b) {
-      const long long slab = 1LL * (b + 1) * ooo;  // W elements per c
+      const long long slab = (b + 1) * ooj;  // W elements per c
       const int ncmax = static_cast<int>(std::max(1LL, welems / slab));
       for (int c0 = b; c0 < v; c0 += ncmax) {
         const int nc = std::min(ncmax, v - c0);
@@ -695,7 +699,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     return LNOCC_ENOMEM;
   }
   count_launch();
-  k_batch_tables<<<(v + 127) / 128, 128, 0, s>>>(o, v, welems, dbat, dbat12);
+  k_batch_tables<<<(v + 127) / 128, 128, 0, s>>>(o, v, jp, welems, dbat, dbat12);
 
   // Block energy kernel. Mixed: w and v staged side by side while they fit (nocc <= 28: 182 KB at 28), one
   // value per element up to nocc 37 (203 KB), at most 8 LOs; FP64: w and v or w alone within 200 KB.
@@ -788,9 +792,11 @@ k_tri_table<<<1, 32, 0, s>>>(o, tri);
     return m;
   };
   const int o2 = static_cast<int>(oo);
-  // grouped launches (two per chunk instead of five) where 128-row tiles hold whole a values (kind 1)
-  // and a (y, z) plane is one (nocc 16) or four (nocc 32) 256-column accumulator tiles
-  const bool grouped = bf && (o == 16 || o == 32) && opts.triples_kernel != LNOCC_TK_PER_TERM;
+  const long long oj = 1LL * o * jp;  // W strides: a ooj, i oj, k jp, j 1
+  // grouped launches (two per chunk instead of five): nocc 16 and 32, where 128-row tiles hold whole a values
+  // and a (y, z) plane is one or four 256-column tiles, in gemm.cu; any other nocc from 4 to 32 in triples_gemm.cu
+  const bool grouped = bf && o >= 4 && o <= 32 && opts.triples_kernel != LNOCC_TK_PER_TERM;
+  const Packed* ops_k2[4] = {&TO, &XT2, &XT2, &XT1};
   const Packed* ops_a[4] = {&XT1, &TO, &XT2, &TOT};
   const Packed* ops_b[4] = {&TO, &XT2, &TO, &XT1};
   const int box_ab[4] = {128, 256, 128, 256};
@@ -801,7 +807,7 @@ k_tri_table<<<1, 32, 0, s>>>(o, tri);
     if (chunk_idx++ % chunk_stride != 0) continue;
     const int b = ch.b, c0 = ch.c0, nc = ch.nc;
     const int na = b + 1, Ma = na * o, Ma2 = na * o2;
-    const long long Sc = 1LL * na * ooo;  // W stride of c
+    const long long Sc = na * ooj;  // W stride of c
     const int xb = b * v * o;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!dev_out) {
@@ -810,7 +816,20 @@ k_tri_table<<<1, 32, 0, s>>>(o, tri);
       cudaEventRecord(e0, s);
     }
     // W layout [c - c0][a][i][k][j]; each term is one contraction over K = v + o (d-part, then l-part).
-    if (grouped) {
+    if (grouped && o != 16 && o != 32) {
+      TgSpec g{};
+      g.b = b;
+      g.c0 = c0;
+      g.nc = nc;
+      g.o = o;
+      g.bvo = xb;
+      g.vo = v * o;
+      g.Sc = Sc;
+      g.kind = 1;
+      gemm_grouped_any(ops_a, g, static_cast<float*>(W), Kt, s, dstatus);
+      g.kind = 2;
+      gemm_grouped_any(ops_k2, g, static_cast<float*>(W), Kt, s, dstatus);
+    } else if (grouped) {
       // launch 1, per (c, 128-row tile of (a, x)): sigma1 + sigma2 stored, then sigma3 and sigma5 added
       // (the output maps of the per-term launches below, restricted to one c)
       GrpSpec g{};
@@ -851,37 +870,37 @@ k_tri_table<<<1, 32, 0, s>>>(o, tri);
     // rows (a,i), cols (k,j): (ai|bd) t_kj^cd - t_il^ab (ck|jl) + (ai|cd) t_jk^bd - t_il^ac (bj|kl)
     {
       OutMap m = omap(0.0);
-      m.sm1 = ooo; m.sm0 = oo; m.mdiv = o;
-      m.sn1 = o; m.sn0 = 1; m.ndiv = o;
+      m.sm1 = ooj; m.sm0 = oj; m.mdiv = o;
+      m.sn1 = jp; m.sn0 = 1; m.ndiv = o;
       gemm2_batched(XT1, TO, &XT1, &TOT, dbat12 + ch.tab, nc, Ma, o2, Kt, Kt, m, s, dstatus);
     }
     // sigma3: rows (a,j), cols (c,k,i): (bj|ad) t_ki^cd - t_jl^ba (ck|il)
     {
       OutMap m = omap(1.0);
-      m.sm1 = ooo; m.sm0 = 1; m.mdiv = o;
-      m.sn2 = Sc; m.sn1 = o; m.sn0 = oo; m.ndiv = o; m.ndiv1 = o;
+      m.sm1 = ooj; m.sm0 = 1; m.mdiv = o;
+      m.sn2 = Sc; m.sn1 = jp; m.sn0 = oj; m.ndiv = o; m.ndiv1 = o;
       gemm_off(XT2, xb, TO, c0 * o2, Ma, nc * o2, Kt, m, s, dstatus);
     }
     // sigma4: rows (a,i,k), cols (c,j): t_ik^ad (bj|cd) - (ai|kl) t_jl^bc
     {
       OutMap m = omap(1.0);
-      m.sm2 = ooo; m.sm1 = oo; m.sm0 = o; m.mdiv = o; m.mdiv1 = o;
+      m.sm2 = ooj; m.sm1 = oj; m.sm0 = jp; m.mdiv = o; m.mdiv1 = o;
       m.sn1 = Sc; m.sn0 = 1; m.ndiv = o;
       gemm_off(TO, 0, XT2, xb + c0 * o, Ma2, nc * o, Kt, m, s, dstatus);
     }
     // sigma6: rows (a,i,j), cols (c,k): t_ij^ad (ck|bd) - (ai|jl) t_kl^cb
     {
       OutMap m = omap(1.0);
-      m.sm2 = ooo; m.sm1 = oo; m.sm0 = 1; m.mdiv = o; m.mdiv1 = o;
-      m.sn1 = Sc; m.sn0 = o; m.ndiv = o;
+      m.sm2 = ooj; m.sm1 = oj; m.sm0 = 1; m.mdiv = o; m.mdiv1 = o;
+      m.sn1 = Sc; m.sn0 = jp; m.ndiv = o;
       gemm_off(TO, 0, XT1, xb + c0 * o, Ma2, nc * o, Kt, m, s, dstatus);
     }
     // sigma5 (batched over c): rows (a,k), cols (i,j): (ck|ad) t_ji^bd - t_kl^ca (bj|il)
     // (TOT[b][i][j] = [t_ji^bd | (bj|il)]: j runs fastest in the columns)
     {
       OutMap m = omap(1.0);
-      m.sm1 = ooo; m.sm0 = o; m.mdiv = o;
-      m.sn1 = oo; m.sn0 = 1; m.ndiv = o;
+      m.sm1 = ooj; m.sm0 = jp; m.mdiv = o;
+      m.sn1 = oj; m.sn0 = 1; m.ndiv = o;
       gemm_batched(XT2, TOT, dbat + ch.tab, nc, Ma, o2, Kt, m, s, dstatus);
     }
     }
@@ -895,10 +914,10 @@ k_tri_table<<<1, 32, 0, s>>>(o, tri);
       count_launch();
       if (bf)
         k_t_energy<float><<<dim3(na, nc), 128, 0, s>>>(static_cast<const float*>(W), Sc, b, c0, o, v, eps, t1, ovov,
-                                                       dU, nlo, tpart + 2 * ch.part);
+                                                       dU, nlo, tpart + 2 * ch.part, jp);
       else
         k_t_energy<double><<<dim3(na, nc), 128, 0, s>>>(static_cast<const double*>(W), Sc, b, c0, o, v, eps, t1,
-                                                        ovov, dU, nlo, tpart + 2 * ch.part);
+                                                        ovov, dU, nlo, tpart + 2 * ch.part, jp);
     }
   }
   {

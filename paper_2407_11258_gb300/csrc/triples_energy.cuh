@@ -172,7 +172,7 @@ struct WalkW {
     for (int p = 0; p < P; ++p)
 #pragma unroll
       for (int u = 0; u < kLoads; ++u)
-        if (O > 0 ? i0 + u < O : i0 + u < o) nxt[p][u] = wp[p][(i0 + u) * (O > 0 ? O * O : o * o)];
+        if (O > 0 ? i0 + u < O : i0 + u < o) nxt[p][u] = wp[p][(i0 + u) * (O > 0 ? O * w_row(O) : o * w_row(o))];
   }
   __device__ __forceinline__ void begin(int o) { load(0, o); }
   // f(p, y0, W of pair p, ad[y0]) for every y0
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(O > 0 ? energy_threads(O) : 64, O > 0 ? energy
   const int o2 = o * o, S1 = blk_s1(o), S0 = blk_s0(o), P1 = o | 1, T = blockDim.x, H = (o + P - 1) / P;
   float2* swv = reinterpret_cast<float2*>(smraw);
   float* small = reinterpret_cast<float*>(swv + ((o * S0 + 1) & ~1));
-  const float* Wb = g.W + slot * g.slot_stride + static_cast<long long>(a) * o2 * o;
+  const float* Wb = g.W + slot * g.slot_stride + static_cast<long long>(a) * o2 * w_row(o);
   constexpr int NA = NLG > 0 ? NLG : 1;
   const int hb = threadIdx.x / o, l = threadIdx.x - hb * o;
   const bool own = hb < H;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(O > 0 ? energy_threads(O) : 64, O > 0 ? energy
 #pragma unroll
   for (int p = 0; p < P; ++p) {
     hp[p] = own && hb + p * H < o ? hb + p * H : (own ? hb : 0);
-    walk.wp[p] = Wb + hp[p] * o + l;
+    walk.wp[p] = Wb + hp[p] * w_row(o) + l;
   }
   if (own) walk.begin(o);
   const EnergySmem m = energy_stage(small, g, a, c, o);
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(energy_threads(O), 1) k_t_energy_single(const 
   const int slot = blockIdx.y, a = blockIdx.x, c = g.c0 + slot;
   const long long blk_id = static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x;
   float* sx = reinterpret_cast<float*>(smraw);
-  const float* Wb = g.W + slot * g.slot_stride + static_cast<long long>(a) * o2 * o;
+  const float* Wb = g.W + slot * g.slot_stride + static_cast<long long>(a) * o2 * w_row(o);
   constexpr int NA = NLG > 0 ? NLG : 1;
   CSum r_can{0.f, 0.f}, r_frag{0.f, 0.f};
   const int hb = threadIdx.x / o, l = threadIdx.x - hb * o;
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(energy_threads(O), 1) k_t_energy_single(const 
   for (int p = 0; p < P; ++p) {
     ok[p] = own && hb + p * H < o;
     hp[p] = ok[p] ? hb + p * H : (own ? hb : 0);
-    walk.wp[p] = Wb + hp[p] * o + l;
+    walk.wp[p] = Wb + hp[p] * w_row(o) + l;
   }
   if (own) walk.begin(o);
   const EnergySmem m = energy_stage(sx + ((o * S0 + 3) & ~3), g, a, c, o);

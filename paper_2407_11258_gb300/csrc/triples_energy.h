@@ -11,12 +11,13 @@ constexpr int kMaxStagedOcc = 37;  // one value per element staged
 // Shared-memory strides of a staged block, all odd (conflict-free for lanes along any slot).
 __host__ __device__ constexpr int blk_s1(int o) { return o | 1; }
 __host__ __device__ constexpr int blk_s0(int o) { return (o * blk_s1(o)) | 1; }
+__host__ __device__ constexpr int w_row(int o) { return (o + 3) & ~3; }  // row length of W (16-byte rows)
 __host__ __device__ constexpr int tri_count(int o) { return o * (o + 1) * (o + 2) / 6; }
 // floats of the slices and vectors of one block
 __host__ __device__ constexpr int energy_small_floats(int o) { return 4 * o + 3 * o * (o | 1) + 2 * o; }
 
 struct EnergyArgs {
-  const float* W;             // chunk [slot][a][i][k][j]
+  const float* W;             // chunk [slot][a][i][k][j], rows of w_row(o) elements
   long long slot_stride;
   int b, c0, o, v;
   const double *eps, *t1;
