@@ -370,43 +370,45 @@ int Frag::build_consts(bool bf) {
   // (ov|vv): (kc|bd) as rows (k,b), K (c,d)               [Z_ij^kb]
   {
     c.kb_cd = alloc_packed(static_cast<int>(ov), static_cast<int>(vv), bf);
-    // B_vv packed once as rows (b,d), K = Q
+    // B_vv packed once as rows (b,d), K = Q: both operands of the ladder integrals, and the second of these
     Packed PBvv = alloc_packed(static_cast<int>(vv), N, bf);
     pack(view(Bvv, kOne, kOne, A(static_cast<int>(vv), 1), kOne, kOne, A(N, vv)), PBvv, s);
     // chunks of k: G[k][c][b][d] (FP64 temp) -> packed rows (k,b), K (c,d)
     const long long per_k = v * vv;
     int kc = static_cast<int>(std::max(1LL, std::min<long long>(o, (1LL << 27) / per_k)));
     double* tmp = static_cast<double*>(alloc(static_cast<size_t>(kc) * per_k * 8));
-    if (!tmp) {
+    if (!tmp || oom) {
       set_error("device allocation failed (ovvv chunk)");
       return LNOCC_ENOMEM;
     }
     for (int k0 = 0; k0 < o; k0 += kc) {
       const int nk = std::min(kc, o - k0);
-      contract_packed_b(view(Bov + k0 * v, kOne, kOne, A(nk * v, 1), kOne, kOne, A(N, ov)), PBvv,
-                        static_cast<int>(vv), out_rowmajor(tmp, vv));
+      gemm_off(c.PBov, k0 * v, PBvv, 0, nk * v, static_cast<int>(vv), N, out_rowmajor(tmp, vv), s, dstatus);
       // tmp[k][c][b][d] -> rows (k0+k, b), K (c, d) of the packed operand
       pack_rows(view(tmp, kOne, A(nk, per_k), A(v, v), kOne, A(v, vv), A(v, 1)), c.kb_cd, k0 * v, s);
     }
-    // ---- packed ladder integrals V+- from G[a][c][b][d] = (ac|bd), chunks of a
+    // ---- packed ladder integrals V+- from G[a][c][b][d] = (ac|bd), chunks of a. V+- need a <= b only, so a
+    // chunk starting at a0 is contracted with the rows b >= a0 (half of all (ac|bd) over the chunks) and takes
+    // more a as those get fewer; its rows (a, c) are rows of the packed B_vv as they stand.
     c.Vp = alloc_packed(np_v, np_v, bf);
     c.Vm = alloc_packed(std::max(nm_v, 1), std::max(nm_v, 1), bf);
     // G chunks in FP32 on the mixed path (V+- are then split to BF16 hi/lo: FP32 carries more bits
-    // than they keep), FP64 on the FP64 path; chunks of a of about 1 GB
+    // than they keep), FP64 on the FP64 path; chunks of about 1 GB (at least one a)
     const size_t gsz = bf ? 4 : 8;
-    int ac = static_cast<int>(std::max(1LL, std::min<long long>(v, (1LL << 30) / (per_k * static_cast<long long>(gsz)))));
-    void* gtmp = alloc(static_cast<size_t>(ac) * per_k * gsz);
+    const long long gcap = std::max(per_k, std::min<long long>(v * per_k, (1LL << 30) / static_cast<long long>(gsz)));
+    void* gtmp = alloc(static_cast<size_t>(gcap) * gsz);
     if (!gtmp || oom) {
       set_error("device allocation failed (vvvv chunk)");
       return LNOCC_ENOMEM;
     }
-    for (int a0 = 0; a0 < v; a0 += ac) {
-      const int na = std::min(ac, v - a0);
-      OutMap gm = out_rowmajor(bf ? nullptr : static_cast<double*>(gtmp), vv);
+    for (int a0 = 0; a0 < v;) {
+      const int nb = v - a0;
+      const int na = static_cast<int>(std::max(1LL, std::min<long long>(nb, gcap / (vv * nb))));
+      OutMap gm = out_rowmajor(bf ? nullptr : static_cast<double*>(gtmp), 1LL * nb * v);
       if (bf) gm.dst32 = static_cast<float*>(gtmp);
-      contract_packed_b(view(Bvv + static_cast<long long>(a0) * v, kOne, kOne, A(na * v, 1), kOne, kOne, A(N, vv)),
-                        PBvv, static_cast<int>(vv), gm);
+      gemm_off(PBvv, a0 * v, PBvv, a0 * v, na * v, nb * v, N, gm, s, dstatus);
       launch_pack_vvvv(gtmp, bf, a0, na, v, c.Vp, c.Vm, s);
+      a0 += na;
     }
     if (!pool) LN_CUDA(cudaStreamSynchronize(s));
     // the chunk temporaries are released right away
@@ -414,7 +416,7 @@ int Frag::build_consts(bool bf) {
       dev_free(p);
       allocs.erase(std::find(allocs.begin(), allocs.end(), p));
     }
-    device_bytes -= static_cast<long long>(kc) * per_k * 8 + static_cast<long long>(ac) * per_k * static_cast<long long>(gsz) +
+    device_bytes -= static_cast<long long>(kc) * per_k * 8 + gcap * static_cast<long long>(gsz) +
                     static_cast<long long>(vv) * round_up(N, 64) * (bf ? 4 : 8);
   }
   mixed = keep;

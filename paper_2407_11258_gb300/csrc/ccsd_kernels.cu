@@ -403,9 +403,9 @@ __global__ void k_pair_L(const double* ovov, double* L, int o, int v) {
   }
 }
 
-// V+/-[ab][cd] from G[a][c][b][d] = (ac|bd) for rows with a in [a0, a0 + na):
+// V+/-[ab][cd] from G[al][c][b - a0][d] = (a0+al c|b d), b >= a0, for rows with a in [a0, a0 + na):
 //   V+ = (ac|bd) + (ad|bc) (a<=b, c<=d),  V- = (ac|bd) - (ad|bc) (a<b, c<d)
-// V+-[ab][cd] from G[al][c][b][d] = (a0+al c|b d): for fixed (al, b) the v x v slice M[c][d] is combined
+// For fixed (al, b) the v x v slice M[c][d] is combined
 // with its transpose, M[c][d] +- M[d][c]. One block per (al, b, 32 x 32 tile pair (cb <= db)): both tiles
 // are read coalesced into shared memory, and the packed rows (c fastest for fixed d, as tri_le(c, d)
 // runs) are written coalesced.
@@ -419,7 +419,7 @@ template <bool BF16, typename TG>
 __global__ void k_pack_vvvv(const TG* __restrict__ G, int a0, int v, void* Vp, void* Vm, int Kpp, int Kpm,
                             long long plane_p, long long plane_m) {
   __shared__ TG T1[32][33], T2[32][33];  // T1[c][d] = M[cb+c][db+d], T2[d][c] = M[db+d][cb+c]
-  const int al = blockIdx.z, b = blockIdx.y, a = a0 + al;
+  const int al = blockIdx.z, b = a0 + blockIdx.y, a = a0 + al;
   if (a > b) return;
   // tile pair index -> (cb, db) with cb <= db over T = ceil(v / 32) tiles
   int tp = blockIdx.x, cbt = 0;
@@ -429,14 +429,14 @@ __global__ void k_pack_vvvv(const TG* __restrict__ G, int a0, int v, void* Vp, v
     ++cbt;
   }
   const int cb = 32 * cbt, db = 32 * (cbt + tp);
-  const long long vv = static_cast<long long>(v) * v;
-  const TG* Mb = G + (static_cast<long long>(al) * v * vv + b * static_cast<long long>(v));  // M[c][d] = Mb[c*vv + d]
+  const long long ldc = static_cast<long long>(v - a0) * v;
+  const TG* Mb = G + (al * v * ldc + blockIdx.y * static_cast<long long>(v));  // M[c][d] = Mb[c*ldc + d]
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;  // 32 x 8
   for (int r = ty; r < 32; r += 8) {
     const int c1 = cb + r, d1 = db + tx;
-    T1[r][tx] = (c1 < v && d1 < v) ? Mb[c1 * vv + d1] : TG(0);
+    T1[r][tx] = (c1 < v && d1 < v) ? Mb[c1 * ldc + d1] : TG(0);
     const int d2 = db + r, c2 = cb + tx;
-    T2[r][tx] = (d2 < v && c2 < v) ? Mb[d2 * vv + c2] : TG(0);
+    T2[r][tx] = (d2 < v && c2 < v) ? Mb[d2 * ldc + c2] : TG(0);
   }
   __syncthreads();
   const long long rowp = static_cast<long long>(tri_le(a, b)) * Kpp;
@@ -726,7 +726,7 @@ void launch_pair_L(const double* ovov, double* L, int o, int v, cudaStream_t s) 
 void launch_pack_vvvv(const void* G, bool g32, int a0, int na, int v, Packed& Vp, Packed& Vm, cudaStream_t s) {
   const long long pp = 1LL * Vp.rows * Vp.Kp, pm = 1LL * Vm.rows * Vm.Kp;
   const int T = (v + 31) / 32;
-  dim3 grid(T * (T + 1) / 2, v, na);
+  dim3 grid(T * (T + 1) / 2, v - a0, na);
   count_launch();
   if (Vp.bf16 && g32)
     k_pack_vvvv<true, float><<<grid, 256, 0, s>>>(static_cast<const float*>(G), a0, v, Vp.p, Vm.p, Vp.Kp, Vm.Kp, pp, pm);
