@@ -29,16 +29,20 @@ namespace lnocc {
 namespace {
 
 constexpr int kBM = 128, kBK = 32, kStages = 4;
-constexpr int kABytes = 2 * kBM * kBK * 2;            // hi and lo planes
-constexpr int kStageBytes = kABytes + 2 * 256 * kBK * 2;
-constexpr int kBoxBytes = kBM * 32 * 4;               // one box of W: 128 rows of at most 32 floats
-constexpr int kSmem = kStages * kStageBytes + 2 * kBoxBytes + 1024 + 256;
-static_assert(kSmem <= 232448, "grouped (T) pipeline does not fit shared memory");
+constexpr int kABytes = 2 * kBM * kBK * 2;  // hi and lo planes
+constexpr int kSmem = 232448;               // all a CTA may hold: four operand stages, the rest boxes of W
+constexpr int kSmemBoxes = kSmem - 1024 - 256;
+constexpr int kMaxBoxes = 4;  // more gain nothing: (19, 125, 500) 36.5, 33.8, 32.7, 32.7 ms per (T) call with 2, 3, 4, 8
+// B planes of N rows after the A planes; at N = 256 and the largest box (128 rows of 32 floats) two boxes fit
+constexpr int stage_bytes(int N) { return kABytes + 2 * N * kBK * 2; }
+static_assert(kSmemBoxes - kStages * stage_bytes(256) >= 2 * kBM * 32 * 4, "grouped (T) pipeline does not fit");
 
 struct TgArgs {
   TgSpec g;
   int rows;     // valid rows of a tile, ta * o
   int N;        // MMA width
+  int stage;    // bytes of an operand stage
+  int box, nbox;  // bytes of a box (a multiple of 128) and how many there are, 2 to kMaxBoxes
   int* status;
 };
 
@@ -97,7 +101,15 @@ __device__ __forceinline__ const CUtensorMap* pick(int id, const CUtensorMap* m0
 __device__ __forceinline__ uint32_t idesc_n(int N) {  // idesc_bf16_f32 for a width known at run time
   return (idesc_bf16_f32(kBM, 0)) | (static_cast<uint32_t>(N >> 3) << 17);
 }
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// At most n copies of this thread still reading their boxes.
+__device__ __forceinline__ void bulk_wait_read(int n) {
+  if (n >= 2)
+    asm volatile("cp.async.bulk.wait_group.read 2;" ::: "memory");
+  else if (n == 1)
+    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+  else
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 // The same barrier with a vote: true when every epilogue thread passes true.
 __device__ __forceinline__ bool epi_all(bool x) {
@@ -120,8 +132,8 @@ __global__ void __launch_bounds__(256, 1)
               const __grid_constant__ CUtensorMap tW0, const __grid_constant__ CUtensorMap tW1, const TgArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* boxes = smem + kStages * kStageBytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(boxes + 2 * kBoxBytes);
+  uint8_t* boxes = smem + kStages * p.stage;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kSmemBoxes);
   uint64_t* empty = full + kStages;
   uint64_t* accf = empty + kStages;
   uint64_t* acce = accf + 2;
@@ -163,7 +175,7 @@ __global__ void __launch_bounds__(256, 1)
           ok = false;
           break;
         }
-        uint8_t* st = smem + s * kStageBytes;
+        uint8_t* st = smem + s * p.stage;
         mbar_arrive_expect_tx(&full[s], bytes);
         const bool s0 = kb < g.nkb;
         const int kc = (s0 ? kb : kb - g.nkb) * kBK;
@@ -194,7 +206,7 @@ __global__ void __launch_bounds__(256, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t a = smem_u32(smem + s * kStageBytes), b = a + kABytes;
+        const uint32_t a = smem_u32(smem + s * p.stage), b = a + kABytes;
 #pragma unroll
         for (int kk = 0; kk < kBK / 16; ++kk) {
           const uint32_t off = kk * 32;
@@ -232,10 +244,10 @@ __global__ void __launch_bounds__(256, 1)
       const uint32_t acc = tmem + buf * 256 + (static_cast<uint32_t>(ew * 32) << 16);
       if (lead && g.kind == 1 && t.term == 1 && t.out0 == 0) bulk_wait_all();  // the region's stores come first
 #pragma unroll 1
-      for (int x = 0; x < t.nout; ++x, ++nbox) {
+      for (int x = 0; x < t.nout; ++x, nbox = nbox + 1 == p.nbox ? 0 : nbox + 1) {
         float v[32];
         tmem_ld32(acc + x * g.o, v);
-        const uint32_t box = box0 + (nbox & 1) * kBoxBytes;
+        const uint32_t box = box0 + nbox * p.box;
         if (rok) {
           if (t.term != 1) {
 #pragma unroll
@@ -248,8 +260,8 @@ __global__ void __launch_bounds__(256, 1)
           }
         }
         fence_proxy_async();
-        // the copy sent from the other box has been read before anybody writes there again
-        if (lead) bulk_wait_read0();
+        // the copy sent from the next box has been read before anybody writes there again
+        if (lead) bulk_wait_read(p.nbox - 2);
         epi_barrier();
         if (lead) {
           const int out = t.out0 + x;
@@ -313,6 +325,9 @@ void gemm_grouped_any(const Packed* const ops[4], TgSpec g, float* W, int K, cud
   a.g = g;
   a.rows = g.ta * g.o;
   a.N = round_up(g.nk * g.o, 16);
+  a.stage = stage_bytes(a.N);
+  a.box = round_up(a.rows * g.jp * 4, 128);
+  a.nbox = std::min(kMaxBoxes, (kSmemBoxes - kStages * a.stage) / a.box);
   a.status = dstatus;
   CUtensorMap m[4], w0, w1;
   for (int k = 0; k < 4; ++k) {
