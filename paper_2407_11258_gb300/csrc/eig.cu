@@ -3,8 +3,9 @@
 // A sweep visits every pair (p, q) once in m - 1 rounds of the round-robin ("circle") schedule over
 // m = n rounded up to even players: in round r, pair 0 is (m - 1, r) and pair k >= 1 is
 // ((r + k) mod (m - 1), (r - k) mod (m - 1)). The m / 2 pairs of one round are disjoint, so their plane
-// rotations commute: one kernel computes the angles that zero every A_pq of the round, a second applies
-// A <- J^T A J as independent 2 x 2 blocks (rows of pair P, columns of pair Q) and V <- V J. A player
+// rotations commute: every A_pq of the round is zeroed at once, A <- J^T A J as independent 2 x 2 blocks (rows of
+// pair P, columns of pair Q) and V <- V J. One cooperative kernel runs a whole sweep with a grid barrier
+// between rounds (k_jac_sweep). A player
 // index >= n (odd n) is a bye. Rotation angles follow the classical form: theta = (A_qq - A_pp) / 2A_pq,
 // t = sgn(theta) / (|theta| + sqrt(theta^2 + 1)), c = 1 / sqrt(1 + t^2), s = t c, which gives
 // A'_pp = A_pp - t A_pq, A'_qq = A_qq + t A_pq, A'_pq = 0. After each sweep the off-diagonal norm is read
@@ -14,9 +15,11 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace lnocc {
 namespace {
@@ -32,15 +35,14 @@ __device__ __forceinline__ void jac_pair(int r, int k, int m, int* p, int* q) {
   }
 }
 
-__global__ void k_jac_angles(const double* __restrict__ A, int n, int m, int r, double2* __restrict__ cs) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= m / 2) return;
+// Rotation that zeroes A_pq of pair k in round r (identity for a bye or a negligible element).
+__device__ __forceinline__ double2 jac_angle(const double* A, int n, int m, int r, int k) {
   int p, q;
   jac_pair(r, k, m, &p, &q);
   double c = 1.0, s = 0.0;
   if (p < n && q < n) {
-    const double apq = A[static_cast<long long>(p) * n + q];
-    const double app = A[static_cast<long long>(p) * n + p], aqq = A[static_cast<long long>(q) * n + q];
+    const double apq = __ldcg(A + static_cast<long long>(p) * n + q);
+    const double app = __ldcg(A + static_cast<long long>(p) * n + p), aqq = __ldcg(A + static_cast<long long>(q) * n + q);
     // skip a rotation whose off-diagonal element is negligible against its diagonal pair
     if (fabs(apq) > 1e-300 && fabs(apq) > 1e-18 * sqrt(fabs(app * aqq))) {
       const double th = (aqq - app) / (2.0 * apq);
@@ -49,50 +51,92 @@ __global__ void k_jac_angles(const double* __restrict__ A, int n, int m, int r, 
       s = t * c;
     }
   }
-  cs[k] = make_double2(c, s);
+  return make_double2(c, s);
 }
 
-// Work items: (m/2)^2 blocks of A, then n * (m/2) row-pairs of V.
-__global__ void k_jac_rotate(double* __restrict__ A, double* __restrict__ V, int n, int m, int r,
-                             const double2* __restrict__ cs) {
-  const long long h = m / 2;
-  const long long nA = h * h, nV = static_cast<long long>(n) * h;
-  for (long long w = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; w < nA + nV;
-       w += static_cast<long long>(gridDim.x) * blockDim.x) {
-    if (w < nA) {
-      const int kP = static_cast<int>(w / h), kQ = static_cast<int>(w % h);
-      int p1, q1, p2, q2;
-      jac_pair(r, kP, m, &p1, &q1);
-      jac_pair(r, kQ, m, &p2, &q2);
-      const double2 g1 = cs[kP], g2 = cs[kQ];
-      const bool r1 = p1 < n, r2 = q1 < n, c1 = p2 < n, c2 = q2 < n;  // byes are absent rows / columns
-      const double a = (r1 && c1) ? A[static_cast<long long>(p1) * n + p2] : 0.0;
-      const double b = (r1 && c2) ? A[static_cast<long long>(p1) * n + q2] : 0.0;
-      const double cc = (r2 && c1) ? A[static_cast<long long>(q1) * n + p2] : 0.0;
-      const double d = (r2 && c2) ? A[static_cast<long long>(q1) * n + q2] : 0.0;
-      // rows: p <- c row_p - s row_q, q <- s row_p + c row_q
-      const double a1 = g1.x * a - g1.y * cc, b1 = g1.x * b - g1.y * d;
-      const double c1v = g1.y * a + g1.x * cc, d1 = g1.y * b + g1.x * d;
-      // columns: p <- c col_p - s col_q, q <- s col_p + c col_q
-      double a2 = g2.x * a1 - g2.y * b1, b2 = g2.y * a1 + g2.x * b1;
-      double c2v = g2.x * c1v - g2.y * d1, d2 = g2.y * c1v + g2.x * d1;
-      if (kP == kQ) b2 = c2v = 0.0;  // the element this rotation annihilates
-      if (r1 && c1) A[static_cast<long long>(p1) * n + p2] = a2;
-      if (r1 && c2) A[static_cast<long long>(p1) * n + q2] = b2;
-      if (r2 && c1) A[static_cast<long long>(q1) * n + p2] = c2v;
-      if (r2 && c2) A[static_cast<long long>(q1) * n + q2] = d2;
-    } else {
-      const long long x = w - nA;
-      const int i = static_cast<int>(x / h), k = static_cast<int>(x % h);
-      int p, q;
-      jac_pair(r, k, m, &p, &q);
-      if (p >= n || q >= n) continue;
-      const double2 g = cs[k];
-      double* row = V + static_cast<long long>(i) * n;
-      const double vp = row[p], vq = row[q];
-      row[p] = g.x * vp - g.y * vq;
-      row[q] = g.y * vp + g.x * vq;
+// All blocks of the grid arrive and wait for each other (cooperative launch: all are resident). The wait has a
+// wall-clock budget; when it runs out the flag is set and every block returns.
+__device__ bool jac_barrier(unsigned* count, unsigned target, int* flag) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    const unsigned long long t0 = globaltimer();
+    ok = 1;
+    unsigned n = 0;
+    while (true) {
+      unsigned c;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
+      if (c >= target) break;
+      if ((++n & 63u) == 0 && globaltimer() - t0 > kWaitBudgetNs) {
+        ok = 0;
+        atomicExch(flag, 1);
+        break;
+      }
     }
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// One sweep of m - 1 rounds, reading A and writing A in turn from one buffer into the other (rounds of even
+// index read A0), V in place. Block (x, y) owns the row pairs [x tP, ...) and column pairs [y tQ, ...) of A and
+// the rows [x tV, ...) of V for the same column pairs, and computes the tP + tQ angles that takes from the old
+// matrix. What others wrote in the round before is read past L1 (__ldcg). Bound by latency: a round is one
+// dependent chain (three elements from L2, a square root and two divisions in FP64, the barrier). With two
+// launches per round (angles, rotations) a round took 10 us; the 1471 rounds of three matrices of order 160, 100
+// and 16 and three small ones fell from 15 to 8.8 ms. (t = 2 a_pq / (|d| + sqrt(d^2 + 4 a_pq^2)) would shorten
+// the chain, but the zero eigenvalues of rank-deficient LO sets then come out as rounding noise.)
+__global__ void __launch_bounds__(256) k_jac_sweep(double* A0, double* A1, double* V, int n, int m, int tP, int tQ,
+                                                   int tV, unsigned* count, int* flag) {
+  extern __shared__ double2 ang[];  // tP row pairs, then tQ column pairs
+  const int h = m / 2, nblk = gridDim.x * gridDim.y;
+  const int p0 = blockIdx.x * tP, np = min(tP, h - p0), q0 = blockIdx.y * tQ, nq = min(tQ, h - q0);
+  const int v0 = blockIdx.x * tV, nv = min(tV, n - v0);
+  for (int r = 0; r < m - 1; ++r) {
+    const double* A = (r & 1) ? A1 : A0;
+    double* B = (r & 1) ? A0 : A1;
+    for (int x = threadIdx.x; x < np + nq; x += blockDim.x)
+      ang[x] = jac_angle(A, n, m, r, x < np ? p0 + x : q0 + x - np);
+    __syncthreads();
+    const int nA = np > 0 && nq > 0 ? np * nq : 0, nV = nv > 0 && nq > 0 ? nv * nq : 0;
+    for (int w = threadIdx.x; w < nA + nV; w += blockDim.x) {
+      if (w < nA) {
+        const int kP = p0 + w / nq, kQ = q0 + w % nq;
+        int p1, q1, p2, q2;
+        jac_pair(r, kP, m, &p1, &q1);
+        jac_pair(r, kQ, m, &p2, &q2);
+        const double2 g1 = ang[w / nq], g2 = ang[np + w % nq];
+        const bool r1 = p1 < n, r2 = q1 < n, c1 = p2 < n, c2 = q2 < n;  // byes are absent rows / columns
+        const double a = (r1 && c1) ? __ldcg(A + static_cast<long long>(p1) * n + p2) : 0.0;
+        const double b = (r1 && c2) ? __ldcg(A + static_cast<long long>(p1) * n + q2) : 0.0;
+        const double cc = (r2 && c1) ? __ldcg(A + static_cast<long long>(q1) * n + p2) : 0.0;
+        const double d = (r2 && c2) ? __ldcg(A + static_cast<long long>(q1) * n + q2) : 0.0;
+        // rows: p <- c row_p - s row_q, q <- s row_p + c row_q
+        const double a1 = g1.x * a - g1.y * cc, b1 = g1.x * b - g1.y * d;
+        const double c1v = g1.y * a + g1.x * cc, d1 = g1.y * b + g1.x * d;
+        // columns: p <- c col_p - s col_q, q <- s col_p + c col_q
+        double a2 = g2.x * a1 - g2.y * b1, b2 = g2.y * a1 + g2.x * b1;
+        double c2v = g2.x * c1v - g2.y * d1, d2 = g2.y * c1v + g2.x * d1;
+        if (kP == kQ) b2 = c2v = 0.0;  // the element this rotation annihilates
+        if (r1 && c1) B[static_cast<long long>(p1) * n + p2] = a2;
+        if (r1 && c2) B[static_cast<long long>(p1) * n + q2] = b2;
+        if (r2 && c1) B[static_cast<long long>(q1) * n + p2] = c2v;
+        if (r2 && c2) B[static_cast<long long>(q1) * n + q2] = d2;
+      } else {
+        const int x = w - nA;
+        int p, q;
+        jac_pair(r, q0 + x % nq, m, &p, &q);
+        if (p >= n || q >= n) continue;
+        const double2 g = ang[np + x % nq];
+        double* row = V + static_cast<long long>(v0 + x / nq) * n;
+        const double vp = __ldcg(row + p), vq = __ldcg(row + q);
+        row[p] = g.x * vp - g.y * vq;
+        row[q] = g.y * vp + g.x * vq;
+      }
+    }
+    if (!jac_barrier(count, static_cast<unsigned>(r + 1) * nblk, flag)) return;
   }
 }
 
@@ -193,39 +237,61 @@ int grid_of(long long work, int threads) {
 
 }  // namespace
 
+// Doubles of scratch that sym_eig needs: norms, barrier and flag, then the second copy of the matrix.
+size_t eig_scratch(int n) { return 16 + static_cast<size_t>(n) * n; }
+
 // A [n][n] symmetric (destroyed); on return w [n] holds the eigenvalues (decreasing when desc, else
 // increasing), order [n] their columns in V, and V [n][n] the eigenvectors as columns (A V = V diag).
-// Device pointers; `scratch` holds at least 16 doubles + m/2 double2. Synchronizes `s` once per sweep.
+// Device pointers; `scratch` holds eig_scratch(n) doubles. Synchronizes `s` once per sweep.
 int sym_eig(double* A, double* V, double* w, int* order, int n, bool desc, double* scratch, cudaStream_t s,
             int* sweeps_out) {
   if (n < 1 || n > kSortMax) {
     set_error("eigendecomposition: size must be in [1, " + std::to_string(kSortMax) + "]");
     return LNOCC_EINVAL;
   }
-  const int m = n + (n & 1);
+  const int m = n + (n & 1), h = m / 2;
   double* norms = scratch;
-  double2* cs = reinterpret_cast<double2*>(scratch + 16);
+  unsigned* count = reinterpret_cast<unsigned*>(scratch + 4);
+  int* flag = reinterpret_cast<int*>(scratch + 5);
+  double* A2 = scratch + 16;
+  LN_CUDA(cudaMemsetAsync(scratch, 0, 16 * sizeof(double), s));
   count_launch();
   k_identity<<<grid_of(1LL * n * n, 256), 256, 0, s>>>(V, n);
   int sweep = 0;
-  double h[2] = {0.0, 0.0};
+  double hn[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if (n > 1) {
-    const long long work = 1LL * (m / 2) * (m / 2) + 1LL * n * (m / 2);
+    // about one 2 x 2 block or row pair a thread, at most one block per SM (all resident); a grid of tiles
+    // close to square keeps the angles each block needs few
+    const long long work = 1LL * h * h + 1LL * n * h;
+    const int blocks = static_cast<int>(std::max(1LL, std::min<long long>(num_sms(), (work + 255) / 256)));
+    int gx = std::max(1, static_cast<int>(std::sqrt(static_cast<double>(blocks))));
+    gx = std::min(gx, h);
+    const int tP = (h + gx - 1) / gx;
+    gx = (h + tP - 1) / tP;
+    const int gy0 = std::max(1, std::min(h, blocks / gx)), tQ = (h + gy0 - 1) / gy0, gy = (h + tQ - 1) / tQ;
+    int nn = n, mm = m, tPa = tP, tQa = tQ, tV = (n + gx - 1) / gx;
     for (sweep = 0; sweep < 60; ++sweep) {
       count_launch();
       k_jac_norms<<<1, 1024, 0, s>>>(A, n, norms);
-      LN_CUDA(cudaMemcpyAsync(h, norms, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+      LN_CUDA(cudaMemcpyAsync(hn, norms, 6 * sizeof(double), cudaMemcpyDeviceToHost, s));
       LN_CUDA(cudaStreamSynchronize(s));
-      if (!std::isfinite(h[1])) {
+      int timed_out = 0;
+      std::memcpy(&timed_out, &hn[5], sizeof(int));
+      if (timed_out) {
+        set_error("eigendecomposition: device wait timed out");
+        return LNOCC_ETIMEOUT;
+      }
+      if (!std::isfinite(hn[1])) {
         set_error("eigendecomposition: non-finite matrix");
         return LNOCC_ENUMERIC;
       }
-      if (h[0] <= 1e-30 * h[1] || h[0] == 0.0) break;
-      for (int r = 0; r < m - 1; ++r) {
-        count_launch(2);
-        k_jac_angles<<<grid_of(m / 2, 128), 128, 0, s>>>(A, n, m, r, cs);
-        k_jac_rotate<<<grid_of(work, 256), 256, 0, s>>>(A, V, n, m, r, cs);
-      }
+      if (hn[0] <= 1e-30 * hn[1] || hn[0] == 0.0) break;
+      LN_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
+      void* args[] = {&A, &A2, &V, &nn, &mm, &tPa, &tQa, &tV, &count, &flag};
+      count_launch();
+      LN_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_jac_sweep), dim3(gx, gy), dim3(256), args,
+                                          static_cast<size_t>(tP + tQ) * sizeof(double2), s));
+      std::swap(A, A2);  // m - 1 rounds, an odd number
     }
     if (sweep == 60) {
       set_error("eigendecomposition: Jacobi sweeps did not converge");

@@ -26,6 +26,7 @@
 
 namespace lnocc {
 
+size_t eig_scratch(int n);
 int sym_eig(double* A, double* V, double* w, int* order, int n, bool desc, double* scratch, cudaStream_t s,
             int* sweeps_out);
 void gather_cols(const double* V, int n, const int* order, int ncols, double* out, int ldo, cudaStream_t s);
@@ -329,7 +330,7 @@ int internal_block(int n, int nlo, const double* U, const double* e, double sv_t
   double* Vg = ar.get_n<double>(1LL * nlo * nlo);
   double* w = ar.get_n<double>(nlo);
   int* ord = ar.get_n<int>(nlo);
-  double* scr = ar.get_n<double>(16 + 2LL * nlo + 8);
+  double* scr = ar.get_n<double>(static_cast<long long>(eig_scratch(nlo)));
   if (ar.failed) {
     set_error("lnocc_lno_internal: device allocation failed");
     return LNOCC_ENOMEM;
@@ -537,7 +538,7 @@ extern "C" int lnocc_lno_select(int n, const double* D, int n_int, const double*
   int* ord = ar.get_n<int>(n);
   int* kord = ar.get_n<int>(n);
   int* cnt = ar.get_n<int>(1);
-  double* scr = ar.get_n<double>(16 + 2LL * n + 8);
+  double* scr = ar.get_n<double>(static_cast<long long>(eig_scratch(n)));
   double* Y = n_int > 0 ? ar.get_n<double>(1LL * n * n_int) : nullptr;
   if (ar.failed) {
     set_error("lnocc_lno_select: device allocation failed");
@@ -593,7 +594,7 @@ extern "C" int lnocc_active_space(int precision, int nocc, int nvir, int naux, c
   double* CF = ar.get_n<double>(1LL * n * nF);
   const int nq_h = static_cast<int>(std::max(1LL, std::min<long long>(N, (1LL << 27) / std::max(1LL * n * round_up(n, 64), 1LL))));
   double* H = ar.get_n<double>(1LL * nq_h * n * nF);
-  double* scr = ar.get_n<double>(16 + 2LL * std::max(no_F, nv_F) + 8);
+  double* scr = ar.get_n<double>(static_cast<long long>(eig_scratch(std::max(no_F, nv_F))));
   if (ar.failed) {
     set_error("lnocc_active_space: device allocation failed");
     return LNOCC_ENOMEM;
