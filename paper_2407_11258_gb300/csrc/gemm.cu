@@ -506,8 +506,7 @@ void splitk_reduce(int splits, int M, int N, const OutMap& C, cudaStream_t s, in
 // pipe (two FMA lanes per clock and SM: 1.1 TFLOP/s over the chip, and 68 us for a single 64 x 64 tile with
 // K = 64 however small the problem).
 void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s, int* dstatus) {
-  (void)K;
-  if (gemm_f64_slices(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, A.Kp, C, false, 0, 0, s,
+  if (gemm_f64_slices(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, K, A.Kp, C, false, 0, 0, s,
                       dstatus))
     return;
   const long long tiles = static_cast<long long>((N + 63) / 64) * ((M + 63) / 64);
@@ -528,7 +527,7 @@ void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s, int* 
   st.launches++;
   st.flops += 1.0 * M * M * A.Kp;  // half of 2 M^2 K
   const double* a = static_cast<const double*>(A.p);
-  if (gemm_f64_slices(a, a, M, M, A.Kp, C, true, 0, 0, s, dstatus)) return;
+  if (gemm_f64_slices(a, a, M, M, A.Kp, A.Kp, C, true, 0, 0, s, dstatus)) return;
   dim3 grid((M + 63) / 64, (M + 63) / 64, 1);
   count_launch();
   k_gemm_f64<true><<<grid, 256, 0, s>>>(a, a, M, M, A.Kp, C, A.Kp, nullptr, nullptr, 0);
@@ -541,7 +540,7 @@ void gemm_f64_lower(const Packed& A, int a_row0, int M, int N, int block, const 
   const double* a0 = a + static_cast<size_t>(a_row0) * A.Kp;
   st.launches++;
   st.flops += 2.0 * M * N * A.Kp;
-  if (gemm_f64_slices(a0, a, M, N, A.Kp, C, false, block, a_row0, s, dstatus)) return;
+  if (gemm_f64_slices(a0, a, M, N, A.Kp, A.Kp, C, false, block, a_row0, s, dstatus)) return;
   Packed A0 = A, B0 = A;
   A0.p = const_cast<double*>(a0);
   gemm_f64(A0, B0, M, N, A.Kp, C, s, dstatus);
@@ -1589,11 +1588,11 @@ void gemm2_batched(const Packed& A0, const Packed& B0, const Packed* A1, const P
     a.batch = dbatch;
     dispatch_tc(A0, B0, A1, B1, a, (maxM + 127) / 128, nbatch, s);
   } else if (A0.sl && B0.sl && (!A1 || (A1->sl && B1->sl))) {
-    gemm_sliced_batched(*A0.sl, *B0.sl, dbatch, nbatch, maxM, N, 0, C, s, dstatus);
+    gemm_sliced_batched(*A0.sl, *B0.sl, dbatch, nbatch, maxM, N, K0, 0, C, s, dstatus);
     if (A1) {
       OutMap C1 = C;
       C1.beta = 1.0;
-      gemm_sliced_batched(*A1->sl, *B1->sl, dbatch, nbatch, maxM, N, 1, C1, s, dstatus);
+      gemm_sliced_batched(*A1->sl, *B1->sl, dbatch, nbatch, maxM, N, K1, 1, C1, s, dstatus);
     }
   } else {
     dim3 grid((maxM + 63) / 64, (N + 63) / 64, nbatch);
@@ -1640,7 +1639,7 @@ void gemm_off(const Packed& A, int a_row0, const Packed& B, int b_row0, int M, i
   if (A.bf16) {
     gemm_tc(A, a_row0, B, b_row0, M, N, C, s, dstatus);
   } else if (A.sl && B.sl) {
-    gemm_sliced(*A.sl, a_row0, *B.sl, b_row0, M, N, C, s, dstatus);
+    gemm_sliced(*A.sl, a_row0, *B.sl, b_row0, M, N, K, C, s, dstatus);
   } else {
     Packed a = A, b = B;
     a.p = static_cast<double*>(A.p) + static_cast<size_t>(a_row0) * A.Kp;

@@ -48,18 +48,29 @@ constexpr int kSmem = kStages * kStageBytes + kTileBytes + 1024 + 256;
 static_assert(kSmem <= 232448, "slices pipeline does not fit shared memory");
 
 // ---------------------------------------------------------------------------------------------
-// Slicing: one warp per (row, chunk), 16 columns per lane, one read of the source.
-__global__ void __launch_bounds__(256) k_slice(const double* __restrict__ src, long long ld, int col0, int rows, int Kp,
-                                               __nv_bfloat16* __restrict__ out, long long plane, int* __restrict__ ex,
-                                               int ex_rows) {
+// Slicing: one warp per (row, chunk), 16 columns per lane, one read of the source. One launch cuts both
+// operands of a product (the items of the second follow those of the first).
+struct SliceJob {
+  const double* src;
+  long long ld;
+  int rows, Kp;
+  __nv_bfloat16* out;
+  int* ex;
+};
+__global__ void __launch_bounds__(256) k_slice(const SliceJob j0, const SliceJob j1) {
   const int lane = threadIdx.x % 32;
-  const int nch = (Kp + kChunk - 1) / kChunk;
-  const long long items = static_cast<long long>(rows) * nch;
+  const long long n0 = static_cast<long long>(j0.rows) * ((j0.Kp + kChunk - 1) / kChunk);
+  const long long items = n0 + static_cast<long long>(j1.rows) * ((j1.Kp + kChunk - 1) / kChunk);
   const long long nw = static_cast<long long>(gridDim.x) * blockDim.x / 32;
-  for (long long it = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) / 32; it < items; it += nw) {
+  for (long long i = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) / 32; i < items; i += nw) {
+    const SliceJob& j = i < n0 ? j0 : j1;
+    const long long it = i < n0 ? i : i - n0, ld = j.ld, plane = static_cast<long long>(j.rows) * j.Kp;
+    const int Kp = j.Kp, ex_rows = j.rows, nch = (Kp + kChunk - 1) / kChunk;
+    int* ex = j.ex;
+    __nv_bfloat16* out = j.out;
     const int r = static_cast<int>(it / nch), ch = static_cast<int>(it % nch);
     const int k0 = ch * kChunk, kw = min(kChunk, Kp - k0);  // kw is a multiple of 64
-    const double* s = src + r * ld + col0 + k0;
+    const double* s = j.src + r * ld + k0;
     double2 x[8];
     unsigned emax = 0, any = 0;
 #pragma unroll
@@ -118,8 +129,8 @@ struct SlArgs {
   int M, N;
   int a_row0, b_row0;       // first rows in the sliced operands
   int mbase, nbase;         // output row / column of local row / column 0
-  int nkb, kper;            // K blocks of 64 of this launch and per work item (kper divides 8)
-  int kblk0;                // first K block (64 columns) in the operands
+  int nkb, kper;            // K blocks of 32 of this launch and per work item (kper divides 16)
+  int kblk0;                // first K block in the operands
   int tiles_m, tiles_n, tiles_z;
   int sym;                  // C = A A^T: tiles on or above the diagonal, mirrored
   int tri, tri_row0;        // tri > 0: only columns n with n / tri <= (tri_row0 + m) / tri are needed
@@ -273,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
     for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
       SlTile ti;
       if (!sl_tile(p, t, ti)) continue;
-      for (int kb = 0; kb < 2 * ti.nkb; ++kb, ++g) {
+      for (int kb = 0; kb < ti.nkb; ++kb, ++g) {
         const int s = g % kStages;
         if (g >= kStages && !mbar_wait(&empty[s], ((g / kStages) - 1) & 1)) {
           atomicExch(p.status, kDevTimeoutProducer);
@@ -282,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
         }
         uint8_t* st = smem + s * kStageBytes;
         mbar_arrive_expect_tx(&full[s], kStageBytes);
-        const int kc = ti.kb0 * 64 + kb * kBK;
+        const int kc = (ti.kb0 + kb) * kBK;
         tma_load_3d(st, &tA, &full[s], kc, ti.a0 + ti.m0, 0);
         tma_load_3d(st + kABytes, &tB, &full[s], kc, ti.b0 + ti.n0, 0);
       }
@@ -299,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
         break;
       }
       tc_fence_after();
-      for (int kb = 0; kb < 2 * ti.nkb; ++kb, ++g) {
+      for (int kb = 0; kb < ti.nkb; ++kb, ++g) {
         const int s = g % kStages;
         if (!mbar_wait(&full[s], (g / kStages) & 1)) {
           atomicExch(p.status, kDevTimeoutMma);
@@ -354,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
       tc_fence_after();
       const int m = ti.m0 + quad * 32 + lane, nbase = ti.n0 + half * 32;
       const bool mok = m < ti.M;
-      const int ch = ti.kb0 / (kChunk / 64);
+      const int ch = ti.kb0 / (kChunk / kBK);
       const int ea = mok ? p.ea[static_cast<long long>(ch) * p.ea_rows + ti.a0 + m] : 0;
       const long long cb = ti.cbase + (p.ws ? static_cast<long long>(ti.z) * p.M * p.N : 0);
       const long long moff = mok ? out_moff(C, mb + m) : 0;
@@ -396,8 +407,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
           if (ea == kBadExp || eb == kBadExp) {
             r[j] = 0.0;
             if (mok && n < p.N) {
-              const double x = sl_dot64(p.A64 + (ti.a0 + m) * p.lda, p.B64 + (ti.b0 + n) * p.ldb, ti.kb0 * 64,
-                                        (ti.kb0 + ti.nkb) * 64);
+              const double x = sl_dot64(p.A64 + (ti.a0 + m) * p.lda, p.B64 + (ti.b0 + n) * p.ldb, ti.kb0 * kBK,
+                                        (ti.kb0 + ti.nkb) * kBK);
               r[j] = p.ws ? x : C.alpha * x;
             }
           } else {
@@ -501,18 +512,24 @@ Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long 
   return s;
 }
 
-void slice(const Sliced& d, cudaStream_t s) {
-  if (d.rows <= 0) return;
-  const long long items = static_cast<long long>(d.rows) * ((d.Kp + kChunk - 1) / kChunk);
-  const int blocks = static_cast<int>(std::min<long long>((items + 7) / 8, 152LL * 16));
-  count_launch();
-  k_slice<<<blocks, 256, 0, s>>>(d.src, d.ld, 0, d.rows, d.Kp, static_cast<__nv_bfloat16*>(d.p),
-                                 static_cast<long long>(d.rows) * d.Kp, d.ex, d.rows);
+static SliceJob slice_job(const Sliced& d) {
+  return SliceJob{d.src, d.ld, d.rows, d.Kp, static_cast<__nv_bfloat16*>(d.p), d.ex};
 }
+static void launch_slice(const Sliced& d, const Sliced* e, cudaStream_t s) {
+  auto items = [](const Sliced& x) { return static_cast<long long>(x.rows) * ((x.Kp + kChunk - 1) / kChunk); };
+  const long long n = items(d) + (e ? items(*e) : 0);
+  if (n <= 0) return;
+  SliceJob j1 = slice_job(d);
+  j1.rows = 0;
+  if (e) j1 = slice_job(*e);
+  count_launch();
+  k_slice<<<static_cast<int>(std::min<long long>((n + 7) / 8, 152LL * 16)), 256, 0, s>>>(slice_job(d), j1);
+}
+void slice(const Sliced& d, cudaStream_t s) { launch_slice(d, nullptr, s); }
 
 // One product of sliced operands (rows from a_row0 / b_row0), K in launches of one chunk unless the
 // partials of several fit the split-K workspace.
-static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C,
+static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, int K, const OutMap& C,
                              int mbase, int nbase, const BatchEntry* batch, int nbatch, int seg, int sym, int tri,
                              int tri_row0, cudaStream_t s, int* dstatus) {
   SlArgs a{};
@@ -531,12 +548,13 @@ static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b
   a.batch = batch;
   a.seg = seg;
   a.status = dstatus;
-  const int nkb = A.Kp / 64;
+  const int nkb = (K + kBK - 1) / kBK;  // columns from K on are zero
   const long long tiles = static_cast<long long>(a.tiles_m) * a.tiles_n, MN = static_cast<long long>(M) * N;
-  constexpr int kcb = kChunk / 64;
-  if (!batch && !sym) {
-    // split K over work items while they do not fill the SMs (a tile of 512 columns takes some 28 us of
-    // MMAs, 64 columns 3.6 us), the FP64 partials summed by the fixed-order reduction
+  constexpr int kcb = kChunk / kBK;
+  if (!batch && !sym && nkb > 5) {
+    // Split K over work items while they do not fill the SMs, the FP64 partials summed by the fixed-order
+    // reduction. A block of 32 columns is 1.8 us of MMAs; up to five of them cost less in one item than the
+    // reduction's launch (about 5 us) and half the MMAs.
     const SplitWs& w = split_ws();
     int kper = kcb;
     while (kper > 1 && tiles * ((nkb + kper - 1) / kper) < num_sms()) kper /= 2;
@@ -563,18 +581,18 @@ static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b
   }
 }
 
-void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C, cudaStream_t s,
-                 int* dstatus) {
-  gemm_sliced_rows(A, a_row0, B, b_row0, M, N, C, 0, 0, nullptr, 1, 0, 0, 0, 0, s, dstatus);
+void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, int K, const OutMap& C,
+                 cudaStream_t s, int* dstatus) {
+  gemm_sliced_rows(A, a_row0, B, b_row0, M, N, K, C, 0, 0, nullptr, 1, 0, 0, 0, 0, s, dstatus);
 }
 
-void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int seg,
-                         const OutMap& C, cudaStream_t s, int* dstatus) {
-  gemm_sliced_rows(A, 0, B, 0, maxM, N, C, 0, 0, dbatch, nbatch, seg, 0, 0, 0, s, dstatus);
+void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int K,
+                         int seg, const OutMap& C, cudaStream_t s, int* dstatus) {
+  gemm_sliced_rows(A, 0, B, 0, maxM, N, K, C, 0, 0, dbatch, nbatch, seg, 0, 0, 0, s, dstatus);
 }
 
 // A (M rows) and B (N rows) packed FP64, K = Kp: slices panels of both into the slice workspace.
-bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, const OutMap& C, bool sym, int tri,
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym, int tri,
                      int tri_row0, cudaStream_t s, int* dstatus) {
   const SplitWs& w = split_ws();
   if (!w.sl || !dstatus) return false;
@@ -586,7 +604,7 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, con
   if (same && bytes(M, Kp) <= w.sl_bytes) {
     const Sliced SA = slice_at(base, M, Kp, A, Kp);
     slice(SA, s);
-    gemm_sliced_rows(SA, 0, SA, 0, M, N, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+    gemm_sliced_rows(SA, 0, SA, 0, M, N, K, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
     return true;
   }
   // the K panel is the whole of K unless even a few row tiles of it would not fit
@@ -595,7 +613,8 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, con
     kp = (kp / 2 + kChunk - 1) / kChunk * kChunk;
   OutMap Ck = C;
   for (int k0 = 0; k0 < Kp; k0 += kp) {
-    const int kw = std::min(kp, Kp - k0);
+    const int kw = std::min(kp, Kp - k0), ku = std::min(kw, K - k0);
+    if (ku <= 0) break;
     // B whole when it leaves room for a quarter of the workspace, else panels of half of it
     const size_t rb = bytes(64, kw);
     int nb = N;
@@ -607,13 +626,14 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, con
       const size_t used = bytes(nn, kw), room = w.sl_bytes - used;
       int mb = M;
       if (bytes(M, kw) > room) mb = std::max(128, static_cast<int>(room / bytes(128, kw)) * 128);
-      slice(SB, s);
+      bool cut_b = true;
       for (int m0 = 0; m0 < M; m0 += mb) {
         const int mm = std::min(mb, M - m0);
         if (sym && n0 + nn <= m0) continue;
         const Sliced SA = slice_at(base + used, mm, kw, A + static_cast<size_t>(m0) * Kp + k0, Kp);
-        slice(SA, s);
-        gemm_sliced_rows(SA, 0, SB, 0, mm, nn, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+        launch_slice(SA, cut_b ? &SB : nullptr, s);
+        cut_b = false;
+        gemm_sliced_rows(SA, 0, SB, 0, mm, nn, ku, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
       }
     }
     Ck.beta = 1.0;

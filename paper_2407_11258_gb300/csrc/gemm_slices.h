@@ -21,14 +21,14 @@ struct Sliced {
 size_t slice_bytes(long long rows, int Kp);  // device bytes of one Sliced operand
 Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long ld);
 void slice(const Sliced& d, cudaStream_t s);  // fill the planes from src
-void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, const OutMap& C, cudaStream_t s,
-                 int* dstatus);
-void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int seg,
-                         const OutMap& C, cudaStream_t s, int* dstatus);
+void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, int K, const OutMap& C,
+                 cudaStream_t s, int* dstatus);
+void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int K,
+                         int seg, const OutMap& C, cudaStream_t s, int* dstatus);
 // C = A B^T for packed FP64 operands through the thread's slice workspace (split_ws().sl): false when
 // there is none (or it is too small): the caller then runs the FP64 SIMT kernel. sym: A == B, the upper
 // part computed and mirrored. tri > 0: only elements with n / tri <= (tri_row0 + m) / tri are needed.
-bool gemm_f64_slices(const double* A, const double* B, int M, int N, int Kp, const OutMap& C, bool sym, int tri,
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym, int tri,
                      int tri_row0, cudaStream_t s, int* dstatus);
 
 }  // namespace lnocc
