@@ -41,9 +41,10 @@ constexpr int kBM = 128, kBN = 64, kBK = 32;
 constexpr int kABytes = kSlices * kBM * kBK * 2, kBBytes = kSlices * kBN * kBK * 2;
 constexpr int kStageBytes = kABytes + kBBytes;  // 96 KB: two stages
 constexpr int kStages = 2;
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;
+constexpr int kEpiCols = kBN / (kEpiWarps / 4);  // columns of one epilogue warp
 constexpr int kThreads = 128 + 32 * kEpiWarps;
-constexpr int kTileBytes = kEpiWarps * 32 * 9 * 8;  // transpose tiles: 32 rows x 8 columns (+1) per warp
+constexpr int kTileBytes = kEpiWarps * 32 * 5 * 8;  // transpose tiles: 32 rows x 4 columns (+1) per warp
 constexpr int kSmem = kStages * kStageBytes + kTileBytes + 1024 + 256;
 static_assert(kSmem <= 232448, "slices pipeline does not fit shared memory");
 
@@ -177,22 +178,22 @@ __device__ __forceinline__ bool sl_tile(const SlArgs& p, int t, SlTile& ti) {
   return ti.m0 < ti.M && ti.nkb > 0;
 }
 
-// 32 lanes x 8 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 32 lanes x 4 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[8][8]) {
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[8][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
   // the loaded values are only defined after the wait: tie them to it
 #pragma unroll
   for (int g = 0; g < 8; ++g)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(v[g][i]));
+    for (int i = 0; i < 4; ++i) asm volatile("" : "+f"(v[g][i]));
 }
 
 // X = hi 2^13 + lo (0 <= lo < 2^13) in units of 2^(-60): the sum of the eight accumulators.
@@ -243,8 +244,9 @@ __device__ __noinline__ double sl_dot64(const double* a, const double* b, int k0
   return acc;
 }
 
-// Persistent: warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4..11 epilogue (two per
-// TMEM lane quadrant, 32 columns each). The eight accumulators of a 128 x 64 tile fill TMEM (8 x 64
+// Persistent: warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4..19 epilogue (four per
+// TMEM lane quadrant, 16 columns each: the accumulators fill TMEM, so the next tile's products wait until all are
+// read; with two warps per quadrant (T) at (8, 64, 256) took 16.6 ms instead of 15.1). The eight accumulators of a 128 x 64 tile fill TMEM (8 x 64
 // columns, accumulator g at column 64 (g - 1)), and the eight B planes sit one after the other in shared
 // memory as 512 rows, so one MMA of N = 256 multiplies plane i of A with four planes of B into four
 // neighbouring accumulators: A is read once per four products.
@@ -345,8 +347,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
       ++it;
     }
   } else if (warp >= 4) {
-    const int ew = warp - 4, quad = ew & 3, half = ew >> 2;
-    double* tile = tiles + ew * (32 * 9);
+    const int ew = warp - 4, quad = ew & 3, part = ew >> 2;
+    double* tile = tiles + ew * (32 * 5);
     const OutMap C = p.ws ? OutMap{p.ws, 0, p.N, 0, 1, 1 << 30, 1 << 30, 1.0, 0.0} : p.C;
     const int mb = p.ws ? 0 : p.mbase, nb = p.ws ? 0 : p.nbase;  // split-K partials are local
     const bool colc = !p.sym && C.sn0 == 1 && !C.dst32;  // columns contiguous: stores go through the transpose tile
@@ -363,39 +365,39 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
       }
       ++it;
       tc_fence_after();
-      const int m = ti.m0 + quad * 32 + lane, nbase = ti.n0 + half * 32;
+      const int m = ti.m0 + quad * 32 + lane, nbase = ti.n0 + part * kEpiCols;
       const bool mok = m < ti.M;
       const int ch = ti.kb0 / (kChunk / kBK);
       const int ea = mok ? p.ea[static_cast<long long>(ch) * p.ea_rows + ti.a0 + m] : 0;
       const long long cb = ti.cbase + (p.ws ? static_cast<long long>(ti.z) * p.M * p.N : 0);
       const long long moff = mok ? out_moff(C, mb + m) : 0;
-      long long roff[8];  // destination rows of the transposed stores
+      long long roff[4];  // destination rows of the transposed stores
       if (colc) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int mm = ti.m0 + quad * 32 + 4 * q + lane / 8;
+        for (int q = 0; q < 4; ++q) {
+          const int mm = ti.m0 + quad * 32 + 8 * q + lane / 4;
           roff[q] = mm < ti.M ? cb + out_moff(C, mb + mm) : -1;
         }
       }
-      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * 32;
+      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * kEpiCols;
 #pragma unroll 1
-      for (int c8 = 0; c8 < 4; ++c8) {
-        float v[8][8];
+      for (int c4 = 0; c4 < kEpiCols / 4; ++c4) {
+        float v[8][4];
 #pragma unroll
-        for (int g = 0; g < 8; ++g) tmem_ld8(acc + g * kBN + 8 * c8, v[g]);
+        for (int g = 0; g < 8; ++g) tmem_ld4(acc + g * kBN + 4 * c4, v[g]);
         tmem_wait_ld(v);
-        if (c8 == 3) {  // everything read: the next tile's products may start
+        if (c4 == kEpiCols / 4 - 1) {  // everything read: the next tile's products may start
           tc_fence_before();
           mbar_arrive(acce);
         }
-        const int n0 = nbase + 8 * c8;
-        if (n0 >= p.N) continue;
-        double r[8];
-        // lane j < 8 holds the exponent of column n0 + j
-        const int nl = n0 + (lane & 7);
+        const int n0 = nbase + 4 * c4;
+        if (n0 >= p.N || ti.m0 + quad * 32 >= ti.M) continue;  // nothing of this warp's is inside
+        double r[4];
+        // lane j < 4 holds the exponent of column n0 + j
+        const int nl = n0 + (lane & 3);
         const int ebl = nl < p.N ? p.eb[static_cast<long long>(ch) * p.eb_rows + ti.b0 + nl] : 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
           const int n = n0 + j;
           const int eb = __shfl_sync(0xffffffffu, ebl, j);
           float a[8];
@@ -432,18 +434,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
         if (colc) {
           __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 8; ++j) tile[lane * 9 + j] = r[j];
+          for (int j = 0; j < 4; ++j) tile[lane * 5 + j] = r[j];
           __syncwarp();
-          const int n = n0 + (lane & 7);
+          const int n = n0 + (lane & 3);
           if (n < p.N) {
             const long long noff = out_noff(C, nb + n);
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              if (roff[q] >= 0) put(roff[q] + noff, tile[(4 * q + lane / 8) * 9 + (lane & 7)]);
+            for (int q = 0; q < 4; ++q)
+              if (roff[q] >= 0) put(roff[q] + noff, tile[(8 * q + lane / 4) * 5 + (lane & 3)]);
           }
         } else if (mok) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < 4; ++j) {
             const int n = n0 + j;
             if (n >= p.N || (p.sym && nb + n < mb + m)) continue;
             put(cb + moff + out_noff(C, nb + n), r[j]);
