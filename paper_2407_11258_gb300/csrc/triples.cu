@@ -644,17 +644,24 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
 
   Sliced sls[4];
   if (tp.slxt > 0) {
+    // without room for the planes the products run on the SIMT kernel from the packed operands
     Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
-    for (int k = 0; k < 4; ++k) {
-      void* mem = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
-      if (!mem) {
-        cleanup();
-        set_error("lnocc_triples: device allocation failed (digit planes)");
-        return LNOCC_ENOMEM;
+    void* mem[4];
+    const size_t n_mine = mine.size();
+    bool room = true;
+    for (int k = 0; k < 4 && room; ++k) {
+      mem[k] = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
+      room = mem[k] != nullptr;
+    }
+    if (room) {
+      for (int k = 0; k < 4; ++k) {
+        sls[k] = slice_at(mem[k], ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
+        slice(sls[k], s);
+        ops[k]->sl = &sls[k];
       }
-      sls[k] = slice_at(mem, ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
-      slice(sls[k], s);
-      ops[k]->sl = &sls[k];
+    } else {
+      for (size_t k = n_mine; k < mine.size(); ++k) dev_free(mine[k]);
+      mine.resize(n_mine);
     }
   }
 
