@@ -642,29 +642,6 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   pack_cols(view(t2, A_(v, 1), A_(v, v), A_(o, o * vv), kOne, kOne, A_(o, vv), -1.0), XT1, 0, v, wl, s);
   pack_cols(view(t2, A_(v, v), A_(v, 1), A_(o, o * vv), kOne, kOne, A_(o, vv), -1.0), XT2, 0, v, wl, s);
 
-  Sliced sls[4];
-  if (tp.slxt > 0) {
-    // without room for the planes the products run on the SIMT kernel from the packed operands
-    Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
-    void* mem[4];
-    const size_t n_mine = mine.size();
-    bool room = true;
-    for (int k = 0; k < 4 && room; ++k) {
-      mem[k] = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
-      room = mem[k] != nullptr;
-    }
-    if (room) {
-      for (int k = 0; k < 4; ++k) {
-        sls[k] = slice_at(mem[k], ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
-        slice(sls[k], s);
-        ops[k]->sl = &sls[k];
-      }
-    } else {
-      for (size_t k = n_mine; k < mine.size(); ++k) dev_free(mine[k]);
-      mine.resize(n_mine);
-    }
-  }
-
   // ---- slabs of fixed b: virtual c in [b, v) in chunks, a in [0, b]; W_chunk[c - c0][a][i][j][k]
   const size_t wsz = bf ? 4 : 8;
   const int jp = tp.jp;
@@ -742,8 +719,31 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     }
     count_launch(2);
     k_ovov_t<<<1216, 256, 0, s>>>(ovov, ovT, o, v);
-k_tri_table<<<1, 32, 0, s>>>(o, tri);
+    k_tri_table<<<1, 32, 0, s>>>(o, tri);
   }
+  Sliced sls[4];
+  if (tp.slxt > 0) {
+    // allocated last: without room for the planes the products run on the SIMT kernel from the packed operands
+    Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
+    void* mem[4];
+    const size_t n_mine = mine.size();
+    bool room = true;
+    for (int k = 0; k < 4 && room; ++k) {
+      mem[k] = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
+      room = mem[k] != nullptr;
+    }
+    if (room) {
+      for (int k = 0; k < 4; ++k) {
+        sls[k] = slice_at(mem[k], ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
+        slice(sls[k], s);
+        ops[k]->sl = &sls[k];
+      }
+    } else {
+      for (size_t k = n_mine; k < mine.size(); ++k) dev_free(mine[k]);
+      mine.resize(n_mine);
+    }
+  }
+
   auto energy_launch = [&](const void* Wp, long long Sc, int b, int c0, int na, int nc, double* part) {
     if (bf) {
       launch_block_energy(EnergyArgs{static_cast<const float*>(Wp), Sc, b, c0, o, v, eps, t1, ovT, dUp, nlo, tri, part, na, nc},
