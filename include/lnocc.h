@@ -45,7 +45,9 @@ extern "C" {
 #define LNOCC_ETIMEOUT 5 /* a bounded device-side wait ran out; results are invalid */
 #define LNOCC_ECUDA 6    /* a CUDA runtime call failed */
 
-#define LNOCC_PREC_FP64 0  /* every contraction in FP64 (plain GPU path) */
+#define LNOCC_PREC_FP64 0  /* every contraction to FP64 accuracy (plain GPU path): products formed from exact BF16
+                              digit products on the tensor pipe and rounded once, errors relative to the
+                              largest elements of the operands' rows */
 #define LNOCC_PREC_MIXED 1 /* contractions as BF16x3 products with FP32 accumulation (tcgen05) */
 
 #define LNOCC_GUESS_MP2 0   /* t1 = 0, t2 = first-order amplitudes (Eq. 21, canonical form) */
@@ -175,7 +177,8 @@ int lnocc_fragment_energy(lnocc_frag* f, int nlo, const double* U_frag, double* 
  *   nlo, U_frag [nocc][nlo] : fragment LO coefficients; U_frag == NULL (or nlo == 0) skips projection.
  *   e_t_full (host)         : canonical (T) energy, the trace of the (T) pair matrix (full active space).
  *   e_t_frag (host)         : sum_alpha sum_ii' U_i,alpha E_ii',(T) U_i',alpha (may be NULL).
- * FP64 precision: FP64 contractions and energy arithmetic. Mixed precision: the W contractions as
+ * FP64 precision: FP64 contractions and energy arithmetic (the digit planes of the contractions' operands,
+ * up to 32 GB, are part of the temporaries). Mixed precision: the W contractions as
  * BF16x3/FP32 on tensor cores; the denominators' terms formed in FP64, the scaled w and v, their
  * products and the i-sums in FP32; a block's partials summed in compensated FP32 (the rounding error
  * of every addition carried alongside, both converted to FP64 once per block) by the staged kernels,
@@ -226,7 +229,7 @@ int lnocc_frag_set_workspace(lnocc_frag* f, void* workspace, long long workspace
 
 /*
  * lnocc_debug_gemm -- diagnostic: C[M][N] = A[M][K] B[N][K]^T through the library's contraction engine
- * (operand packing + FP64 SIMT GEMM, or BF16x3 tcgen05 GEMM with FP32 accumulation). Device pointers,
+ * (operand packing + FP64 digit-plane GEMM, or BF16x3 tcgen05 GEMM with FP32 accumulation). Device pointers,
  * row-major FP64. Allocates its own temporaries and synchronizes `stream`. Not part of the method; it
  * lets the contraction kernels be checked on their own.
  */
