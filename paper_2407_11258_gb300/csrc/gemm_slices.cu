@@ -34,7 +34,6 @@
 namespace lnocc {
 namespace {
 
-constexpr int kSlices = 8;
 constexpr int kChunk = kSliceChunk;     // columns that share an exponent and an exact accumulation
 constexpr int kBadExp = 0x40000000;     // chunk that cannot be sliced
 constexpr int kBM = 128, kBN = 64, kBK = 32;
@@ -496,12 +495,6 @@ void launch_sl(const Sliced& A, const Sliced& B, SlArgs a, cudaStream_t s) {
 
 }  // namespace
 
-size_t slice_bytes(long long rows, int Kp) {
-  const size_t planes = static_cast<size_t>(rows) * Kp * 2 * kSlices;
-  const size_t ex = static_cast<size_t>(rows) * ((Kp + kChunk - 1) / kChunk) * 4;
-  return (planes + 255) / 256 * 256 + (ex + 255) / 256 * 256;
-}
-
 Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long ld) {
   Sliced s;
   s.rows = static_cast<int>(rows);
@@ -598,48 +591,26 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int 
                      int tri_row0, cudaStream_t s, int* dstatus) {
   const SplitWs& w = split_ws();
   if (!w.sl || !dstatus) return false;
-  auto bytes = [](long long rows, int k) { return slice_bytes(rows, k); };
-  if (bytes(std::min(M, 512), std::min(Kp, 2 * kChunk)) + bytes(std::min(N, 256), std::min(Kp, 2 * kChunk)) > w.sl_bytes)
-    return false;
   unsigned char* base = static_cast<unsigned char*>(w.sl);
   const bool same = A == B && M == N;
-  if (same && bytes(M, Kp) <= w.sl_bytes) {
+  if (same && slice_bytes(M, Kp) <= w.sl_bytes) {
     const Sliced SA = slice_at(base, M, Kp, A, Kp);
     slice(SA, s);
     gemm_sliced_rows(SA, 0, SA, 0, M, N, K, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
     return true;
   }
-  // the K panel is the whole of K unless even a few row tiles of it would not fit
-  int kp = Kp;
-  while (kp > 2 * kChunk && bytes(std::min(M, 512), kp) + bytes(std::min(N, 256), kp) > w.sl_bytes)
-    kp = (kp / 2 + kChunk - 1) / kChunk * kChunk;
+  const SlicePanels pl = plan_slice_panels(M, N, Kp, w.sl_bytes);
+  if (pl.kw == 0) return false;
   OutMap Ck = C;
-  for (int k0 = 0; k0 < Kp; k0 += kp) {
-    const int kw = std::min(kp, Kp - k0), ku = std::min(kw, K - k0);
-    if (ku <= 0) break;
-    // B whole when it leaves room for a quarter of the workspace, else panels of half of it
-    const size_t rb = bytes(64, kw);
-    int nb = N;
-    if (bytes(N, kw) > w.sl_bytes / 4 * 3 && bytes(N, kw) + bytes(M, kw) > w.sl_bytes)
-      nb = std::max(64, static_cast<int>(w.sl_bytes / 2 / rb) * 64);
-    for (int n0 = 0; n0 < N; n0 += nb) {
-      const int nn = std::min(nb, N - n0);
-      const Sliced SB = slice_at(base, nn, kw, B + static_cast<size_t>(n0) * Kp + k0, Kp);
-      const size_t used = bytes(nn, kw), room = w.sl_bytes - used;
-      int mb = M;
-      if (bytes(M, kw) > room) mb = std::max(128, static_cast<int>(room / bytes(128, kw)) * 128);
-      bool cut_b = true;
-      for (int m0 = 0; m0 < M; m0 += mb) {
-        const int mm = std::min(mb, M - m0);
-        if (sym && n0 + nn <= m0) continue;
-        const Sliced SA = slice_at(base + used, mm, kw, A + static_cast<size_t>(m0) * Kp + k0, Kp);
-        launch_slice(SA, cut_b ? &SB : nullptr, s);
-        cut_b = false;
-        gemm_sliced_rows(SA, 0, SB, 0, mm, nn, ku, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
-      }
-    }
-    Ck.beta = 1.0;
-  }
+  for_each_slice_panel(pl, M, N, Kp, sym, [&](int k0, int kw, int n0, int nn, int m0, int mm, bool first) {
+    const int ku = std::min(kw, K - k0);
+    if (ku <= 0) return;
+    const Sliced SB = slice_at(base, nn, kw, B + static_cast<size_t>(n0) * Kp + k0, Kp);
+    const Sliced SA = slice_at(base + slice_bytes(nn, kw), mm, kw, A + static_cast<size_t>(m0) * Kp + k0, Kp);
+    launch_slice(SA, first ? &SB : nullptr, s);
+    Ck.beta = k0 == 0 ? C.beta : 1.0;
+    gemm_sliced_rows(SA, 0, SB, 0, mm, nn, ku, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+  });
   return true;
 }
 

@@ -3,10 +3,9 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "slice_panels.h"
 
 namespace lnocc {
-
-constexpr int kSliceChunk = 512;  // columns that share one exponent
 
 // Rows of a packed FP64 operand (row stride ld, Kp columns) as eight BF16 planes [8][rows][Kp] and the
 // exponents [ceil(Kp / 512)][rows] of their chunks.
@@ -18,7 +17,6 @@ struct Sliced {
   long long ld = 0;
 };
 
-size_t slice_bytes(long long rows, int Kp);  // device bytes of one Sliced operand
 Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long ld);
 void slice(const Sliced& d, cudaStream_t s);  // fill the planes from src
 void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M, int N, int K, const OutMap& C,
