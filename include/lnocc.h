@@ -45,9 +45,9 @@ extern "C" {
 #define LNOCC_ETIMEOUT 5 /* a bounded device-side wait ran out; results are invalid */
 #define LNOCC_ECUDA 6    /* a CUDA runtime call failed */
 
-#define LNOCC_PREC_FP64 0  /* every contraction to FP64 accuracy (plain GPU path): products formed from exact BF16
-                              digit products on the tensor pipe and rounded once, errors relative to the
-                              largest elements of the operands' rows */
+#define LNOCC_PREC_FP64 0  /* every contraction in FP64 (plain GPU path): exact BF16 digit products on the tensor pipe,
+                              rounded once; elements whose terms are all far below the product of their rows' largest
+                              elements are summed in FP64, so that none is less exact than by an FP64 FMA chain */
 #define LNOCC_PREC_MIXED 1 /* contractions as BF16x3 products with FP32 accumulation (tcgen05) */
 
 #define LNOCC_GUESS_MP2 0   /* t1 = 0, t2 = first-order amplitudes (Eq. 21, canonical form) */

@@ -4,19 +4,25 @@
 // product is formed from exact BF16 products instead, after Ozaki, Ogita, Oishi and Rump (Numer.
 // Algorithms 59, 95 (2012)) and its tensor-core form (Mukunoki et al., ISC 2020):
 //   * Each operand row is cut into chunks of kChunk = 512 columns. A chunk shares one exponent E (all
-//     |x| < 2^E) and every x 2^-E becomes eight balanced radix-128 digits, x = 2^(E-6) sum_i d_i 2^(-7(i-1)),
-//     d_1..d_7 integers in [-64, 64] and the eighth the remainder rounded to BF16; plane i holds
-//     d_i 2^(-7(i-1)), exact in BF16.
-//   * A(m, :) . B(n, :) = 2^(Ea+Eb-12) sum_g S_g with S_g the digit products of i + j = g + 1. One FP32
-//     TMEM accumulator per g = 1..8. For g <= 7 every term is an integer times 2^(-7(g-1)) and
-//     |S_g| <= 7 * 512 * 64 * 64 < 2^24 units, so the accumulation is exact; accumulator 8 also takes the
-//     pairs i + j = 10 (weight 2^-56 against S_1: an FP32 rounding there is below 2^-66).
-//   * The epilogue adds the accumulators as a 72-bit integer and rounds it once to FP64.
-// What is dropped: the pairs i + j > 10 and the operands beyond their 57th bit, both relative to the
-// largest element of their chunk. The error of an element of C is about 0.05 sqrt(K) 2^-56 rowmax colmax,
-// below the K 2^-53 sum|a||b| growth of an FP64 FMA chain on the library's operands.
-// Rows whose chunk holds an infinity, a NaN, or only subnormal values are marked; their outputs are summed
-// in FP64 from the packed operand, so those propagate as in an FP64 product.
+//     |x| < 2^E) and every x 2^-E, rounded to 62 fraction bits, becomes nine balanced radix-128 digits,
+//     x = 2^(E-6) sum_i d_i 2^(-7(i-1)), integers in [-64, 64]; plane i holds d_i 2^(-7(i-1)), exact in BF16.
+//   * A(m, :) . B(n, :) = 2^(Ea+Eb-12) sum_g S_g with S_g the digit products of i + j = g + 1, one FP32 TMEM
+//     accumulator per g = 1..9. Every term of S_g is an integer times 2^(-7(g-1)) and |S_g| <= g 512 64 64 <= 2^24
+//     units for g <= 8, so the accumulation is exact; g = 9 can round at 2^-68 of 2^(Ea+Eb).
+//   * The epilogue adds the accumulators as one integer and rounds it once to FP64.
+// What is dropped is absolute in 2^(Ea+Eb): the pairs i + j > 10, in root mean square sqrt(K) 2^-63.1 (digits
+// uniform, eight pairs of i + j = 11), and the rounding of the operands at 2^-63. An FP64 FMA chain instead errs
+// relative to T = sum |a||b| of the element: at least about 0.6 2^-53 T. So that no element is less exact
+// than by the chain, a tenth plane holds |x| 2^-E, a tenth accumulator sums T, and an element with
+// T < 2^-9 sqrt(K) 2^(Ea+Eb), where the digits would give less, is summed in FP64 from the packed operands.
+// (At that line the digits' error is 0.5 2^-53 T.) T = 0 means that no nonzero meets another: zero exactly.
+// On the library's operands 0 to 0.3% of the elements fall below the line, in two products about half of them
+// (the (k,b) amplitude part of the dressed three-index terms, and the rotation of B into an active space,
+// whose rows decay away from their centre). With eight planes and no such check (128 x 64 tiles) 3 CCSD iterations
+// at (12, 96, 320) took 11.7 instead of 13.8 ms, (T) at (8, 64, 256) 15.1 instead of 18.2 ms (its 64-column products
+// take two tiles now) and the LNO space of (16, 160, 640) 13.9 instead of 21.3 ms (7.3 ms in the two products
+// that fall back), but an element 1e-16 of its row's largest was kept to 6e-3. The SIMT kernel: 131.6, 67.1, 30.4 ms.
+// Rows whose chunk holds an infinity, a NaN, or only subnormal values are marked and summed in FP64 too.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -36,15 +42,15 @@ namespace {
 
 constexpr int kChunk = kSliceChunk;     // columns that share an exponent and an exact accumulation
 constexpr int kBadExp = 0x40000000;     // chunk that cannot be sliced
-constexpr int kBM = 128, kBN = 64, kBK = 32;
-constexpr int kABytes = kSlices * kBM * kBK * 2, kBBytes = kSlices * kBN * kBK * 2;
-constexpr int kStageBytes = kABytes + kBBytes;  // 96 KB: two stages
+constexpr int kBM = 128, kBN = 48, kBK = 32;
+constexpr int kABytes = kPlanes * kBM * kBK * 2, kBBytes = kPlanes * kBN * kBK * 2;
+constexpr int kStageBytes = kABytes + kBBytes;  // 110 KB: two stages
 constexpr int kStages = 2;
 constexpr int kEpiWarps = 16;
-constexpr int kEpiCols = kBN / (kEpiWarps / 4);  // columns of one epilogue warp
+constexpr int kEpiUnits = 2 * (kBN / 8) / (kEpiWarps / 4);  // units of 16 rows x 8 columns of one epilogue warp
 constexpr int kThreads = 128 + 32 * kEpiWarps;
-constexpr int kTileBytes = kEpiWarps * 32 * 5 * 8;  // transpose tiles: 32 rows x 4 columns (+1) per warp
-constexpr int kSmem = kStages * kStageBytes + kTileBytes + 1024 + 256;
+constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
+static_assert((kSlices + 1) * kBN <= 512 && 2 * (kBN / 8) % (kEpiWarps / 4) == 0, "accumulators, epilogue split");
 static_assert(kSmem <= 232448, "slices pipeline does not fit shared memory");
 
 // ---------------------------------------------------------------------------------------------
@@ -88,27 +94,30 @@ __global__ void __launch_bounds__(256) k_slice(const SliceJob j0, const SliceJob
     if (lane == 0) ex[static_cast<long long>(ch) * ex_rows + r] = bad ? kBadExp : static_cast<int>(emax) - 1022;
     __nv_bfloat16* o = out + static_cast<long long>(r) * Kp + k0;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const int k = 2 * (lane + 32 * t);
+    for (int q = 0; q < 8; ++q) {
+      const int k = 2 * (lane + 32 * q);
       if (k >= kw) break;
-      long long F[2];  // x 2^-E with 61 fraction bits
+      long long F[2];  // x 2^-E with 62 fraction bits, rounded
+      float t[2];      // |x| 2^-E; a nonzero keeps at least 2^-60, so that no product of two of them is lost
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const long long u = __double_as_longlong(h ? x[t].y : x[t].x);
+        const long long u = __double_as_longlong(h ? x[q].y : x[q].x);
         const int e = static_cast<int>(u >> 52) & 0x7ff;
         long long m = (u & 0xfffffffffffffLL) | (e > 0 ? 0x10000000000000LL : 0);
-        const int sh = static_cast<int>(emax) + 1 - max(e, 1);  // >= 1
-        m = sh <= 9 ? m << (9 - sh) : (sh < 64 ? m >> (sh - 9) : 0);
+        const int sh = static_cast<int>(emax) + 1 - max(e, 1);  // >= 1: x 2^-E = m 2^(-52 - sh)
+        const float a = m == 0 ? 0.f : fmaxf(static_cast<float>(m >> 24) * __int_as_float((127 - 28 - min(sh, 60)) << 23), 0x1p-60f);
+        m = sh <= 10 ? m << (10 - sh) : (sh < 65 ? (m + (1LL << (sh - 11))) >> (sh - 10) : 0);
         F[h] = bad ? 0 : (u < 0 ? -m : m);
+        t[h] = bad ? 0.f : a;
       }
       float w = 1.f;
 #pragma unroll
-      for (int i = 1; i <= 7; ++i) {
-        const int sft = 62 - 7 * i;
+      for (int i = 1; i <= kSlices; ++i) {
+        const int sft = 63 - 7 * i;
         float f[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const long long d = (F[h] + (1LL << (sft - 1))) >> sft;
+          const long long d = sft > 0 ? (F[h] + (1LL << (sft > 0 ? sft - 1 : 0))) >> sft : F[h];
           F[h] -= d << sft;
           // d in [-64, 64] to FP32 through the exponent of 1.5 2^23, scaled by the plane's weight (exact)
           const float g = __int_as_float(0x4B400000 + static_cast<int>(d));
@@ -117,9 +126,7 @@ __global__ void __launch_bounds__(256) k_slice(const SliceJob j0, const SliceJob
         *reinterpret_cast<__nv_bfloat162*>(o + (i - 1) * plane + k) = __floats2bfloat162_rn(f[0], f[1]);
         w *= 0.0078125f;
       }
-      // |F| <= 2^12 here: the eighth plane holds F 2^-55 rounded to BF16
-      *reinterpret_cast<__nv_bfloat162*>(o + 7 * plane + k) = __floats2bfloat162_rn(
-          static_cast<float>(static_cast<int>(F[0])) * 0x1p-55f, static_cast<float>(static_cast<int>(F[1])) * 0x1p-55f);
+      *reinterpret_cast<__nv_bfloat162*>(o + kSlices * plane + k) = __floats2bfloat162_rn(t[0], t[1]);
     }
   }
 }
@@ -136,7 +143,7 @@ struct SlArgs {
   int tri, tri_row0;        // tri > 0: only columns n with n / tri <= (tri_row0 + m) / tri are needed
   const int *ea, *eb;       // chunk exponents [chunk][rows]
   int ea_rows, eb_rows;
-  const double *A64, *B64;  // the packed FP64 operands (rows as a_row0 / b_row0), for marked chunks
+  const double *A64, *B64;  // the packed FP64 operands (rows as a_row0 / b_row0), for elements summed in FP64
   long long lda, ldb;
   int asign, ashift;        // alpha = asign 2^ashift when asign != 0, else C.alpha multiplies
   OutMap C;
@@ -177,51 +184,52 @@ __device__ __forceinline__ bool sl_tile(const SlArgs& p, int t, SlTile& ti) {
   return ti.m0 < ti.M && ti.nkb > 0;
 }
 
-// 32 lanes x 4 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+// 16 lanes x 8 columns: lane l of the warp gets (row l / 4, columns 2 (l % 4), + 1), then the same of row l / 4 + 8.
+__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, float (&v)[4]) {
   uint32_t r[4];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 #pragma unroll
   for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_wait_ld(float (&v)[8][4]) {
+__device__ __forceinline__ void tmem_wait_ld(float (&v)[kSlices + 1][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
   // the loaded values are only defined after the wait: tie them to it
 #pragma unroll
-  for (int g = 0; g < 8; ++g)
+  for (int g = 0; g <= kSlices; ++g)
 #pragma unroll
     for (int i = 0; i < 4; ++i) asm volatile("" : "+f"(v[g][i]));
 }
 
-// X = hi 2^13 + lo (0 <= lo < 2^13) in units of 2^(-60): the sum of the eight accumulators.
+// X = hi 2^21 + lo (0 <= lo < 2^21) in units of 2^(-68): the sum of the nine accumulators.
 __device__ __forceinline__ void sl_combine(const float* a, long long& hi, int& lo) {
   const int s1 = __float2int_rn(a[0]), s2 = __float2int_rn(a[1] * 0x1p7f), s3 = __float2int_rn(a[2] * 0x1p14f);
   const int s4 = __float2int_rn(a[3] * 0x1p21f), s5 = __float2int_rn(a[4] * 0x1p28f), s6 = __float2int_rn(a[5] * 0x1p35f);
-  // |s1| <= 2^21, |s2| <= 2^22, ...: each pair fits 32 bits
+  // |s1| <= 2^21, |s2| <= 2^22, ..., |s8| <= 2^24: each of these pairs fits 32 bits
   const int p1 = s1 * 128 + s2, p2 = s3 * 128 + s4, p3 = s5 * 128 + s6;
-  const int t = __float2int_rn(a[6] * 0x1p48f) + __float2int_rn(a[7] * 0x1p48f);
-  hi = static_cast<long long>(p1) * (1 << 28) + (static_cast<long long>(p2) * (1 << 14) + p3) + (t >> 13);
-  lo = t & 0x1fff;
+  const int s7 = __float2int_rn(a[6] * 0x1p42f), s8 = __float2int_rn(a[7] * 0x1p49f), s9 = __float2int_rn(a[8] * 0x1p56f);
+  const long long t = static_cast<long long>(s7) * (1 << 14) + (static_cast<long long>(s8) * 128 + s9);
+  hi = static_cast<long long>(p1) * (1 << 28) + (static_cast<long long>(p2) * (1 << 14) + p3) + (t >> 21);
+  lo = static_cast<int>(t & 0x1fffff);
 }
 
-// (hi 2^13 + lo) 2^(e-60) rounded once to FP64; neg flips the sign.
+// (hi 2^21 + lo) 2^(e-68) rounded once to FP64; neg flips the sign.
 __device__ __forceinline__ double sl_round(long long hi, int lo, int e, bool flip) {
   bool neg = hi < 0;
   if (neg) {
     hi = lo ? ~hi : -hi;
-    lo = (0x2000 - lo) & 0x1fff;
+    lo = (0x200000 - lo) & 0x1fffff;
   }
   unsigned long long m;
   int lz;
   if (hi != 0) {
     lz = __clzll(hi);
     m = (static_cast<unsigned long long>(hi) << lz) |
-        (lz >= 13 ? static_cast<unsigned long long>(lo) << (lz - 13) : static_cast<unsigned long long>(lo) >> (13 - lz));
+        (lz >= 21 ? static_cast<unsigned long long>(lo) << (lz - 21) : static_cast<unsigned long long>(lo) >> (21 - lz));
   } else if (lo != 0) {
-    lz = __clzll(static_cast<long long>(lo)) + 13;
-    m = static_cast<unsigned long long>(lo) << (lz - 13);
+    lz = __clzll(static_cast<long long>(lo)) + 21;
+    m = static_cast<unsigned long long>(lo) << (lz - 21);
   } else {
     return 0.0;
   }
@@ -236,25 +244,57 @@ __device__ __forceinline__ double sl_round(long long hi, int lo, int e, bool fli
   return neg ? -r : r;
 }
 
-// FP64 sum over the work item's columns, for rows whose chunk could not be sliced.
-__device__ __noinline__ double sl_dot64(const double* a, const double* b, int k0, int k1) {
-  double acc = 0.0;
-  for (int k = k0; k < k1; ++k) acc = fma(a[k], b[k], acc);
-  return acc;
+// FP64 sums in place of the digits' for the elements of a warp's unit of 16 rows x 8 columns that `need` marks
+// (bit 2 r + c: row r_lane + 8 r, column c_lane + c of this lane's four), from the packed operands' rows
+// (a0, b0: the lane's first ones; 8 lda and ldb further on the others), k columns. Four elements at a
+// time, eight lanes each: FP64-pipe work is k / 8 + 3 instructions per four elements, half of what a walk of every
+// lane over its own four would take when half of the unit is marked, and no more when all is.
+__device__ __noinline__ void sl_dot64(const double* a0, long long lda8, const double* b0, long long ldb, int k, unsigned need,
+                                      double (&r)[4]) {
+  const int lane = threadIdx.x & 31, grp = lane >> 3, sub = lane & 7;
+  unsigned any = __ballot_sync(0xffffffffu, need != 0u);
+  while (any) {
+    // group g takes the first marked element of the g-th marked lane
+    unsigned t = any;
+    for (int q = 0; q < grp; ++q) t &= t - 1;
+    const int src = t ? __ffs(t) - 1 : lane, e = need ? __ffs(need) - 1 : 0;
+    const unsigned long long x = reinterpret_cast<unsigned long long>((e & 2) ? a0 + lda8 : a0);
+    const unsigned long long y = reinterpret_cast<unsigned long long>((e & 1) ? b0 + ldb : b0);
+    const double* xs = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, x, src)) + 2 * sub;
+    const double* ys = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, y, src)) + 2 * sub;
+    double acc = 0.0;
+    if (t) {
+#pragma unroll 4
+      for (int q = 0; q < k; q += 16) {
+        const double2 u = *reinterpret_cast<const double2*>(xs + q), v = *reinterpret_cast<const double2*>(ys + q);
+        acc = fma(u.y, v.y, fma(u.x, v.x, acc));
+      }
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    const int rank = __popc(any & ((1u << lane) - 1u));
+    const double got = __shfl_sync(0xffffffffu, acc, 8 * (rank & 3));
+    if (need && rank < 4) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        if (h == e) r[h] = got;
+      need &= need - 1;
+    }
+    any = __ballot_sync(0xffffffffu, need != 0u);
+  }
 }
 
-// Persistent: warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4..19 epilogue (four per
-// TMEM lane quadrant, 16 columns each: the accumulators fill TMEM, so the next tile's products wait until all are
-// read; with two warps per quadrant (T) at (8, 64, 256) took 16.6 ms instead of 15.1). The eight accumulators of a 128 x 64 tile fill TMEM (8 x 64
-// columns, accumulator g at column 64 (g - 1)), and the eight B planes sit one after the other in shared
-// memory as 512 rows, so one MMA of N = 256 multiplies plane i of A with four planes of B into four
-// neighbouring accumulators: A is read once per four products.
+// Persistent: warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4..19 epilogue (four per TMEM lane
+// quadrant: the accumulators nearly fill TMEM, so the next tile's products wait until all are read). The ten
+// accumulators of a 128 x 48 tile take 480 TMEM columns (accumulator g at column 48 (g - 1), T last), and the
+// digit planes of B sit one after the other in shared memory as 432 rows, so one MMA of N = 240 multiplies
+// plane i of A with five planes of B into five neighbouring accumulators: A is read once per five products.
 __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__ CUtensorMap tA,
                                                          const __grid_constant__ CUtensorMap tB, const SlArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  double* tiles = reinterpret_cast<double*>(smem + kStages * kStageBytes);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes + kTileBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
   uint64_t* empty = full + kStages;
   uint64_t* accf = empty + kStages;
   uint64_t* acce = accf + 1;
@@ -326,19 +366,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
           const uint32_t first = (kb | kk) != 0 ? 1u : 0u;
 #pragma unroll
           for (int i = 0; i < kSlices; ++i) {
-            // plane i of A against planes 0 .. 7 - i of B: accumulators i .. 7
+            // plane i of A against planes 0 .. 8 - i of B: accumulators i .. 8
             const uint64_t da = sdesc_sw64(a0 + i * (kBM * kBK * 2) + off);
 #pragma unroll
-            for (int j = 0; j < kSlices - i; j += 4) {
-              const int nj = kSlices - i - j < 4 ? kSlices - i - j : 4;
+            for (int j = 0; j < kSlices - i; j += 5) {
+              const int nj = kSlices - i - j < 5 ? kSlices - i - j : 5;
               mma_bf16(tmem + (i + j) * kBN, da, sdesc_sw64(b0 + j * (kBN * kBK * 2) + off),
                        idesc_bf16_f32(kBM, nj * kBN), i == 0 ? first : 1u);
             }
-            // and plane 8 - i: the leading dropped diagonal, into accumulator 7
-            if (i > 0)
-              mma_bf16(tmem + 7 * kBN, da, sdesc_sw64(b0 + (8 - i) * (kBN * kBK * 2) + off),
-                       idesc_bf16_f32(kBM, kBN), 1u);
           }
+          // T
+          mma_bf16(tmem + kSlices * kBN, sdesc_sw64(a0 + kSlices * (kBM * kBK * 2) + off),
+                   sdesc_sw64(b0 + kSlices * (kBN * kBK * 2) + off), idesc_bf16_f32(kBM, kBN), first);
         }
         mma_commit(&empty[s]);
       }
@@ -347,10 +386,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
     }
   } else if (warp >= 4) {
     const int ew = warp - 4, quad = ew & 3, part = ew >> 2;
-    double* tile = tiles + ew * (32 * 5);
     const OutMap C = p.ws ? OutMap{p.ws, 0, p.N, 0, 1, 1 << 30, 1 << 30, 1.0, 0.0} : p.C;
     const int mb = p.ws ? 0 : p.mbase, nb = p.ws ? 0 : p.nbase;  // split-K partials are local
-    const bool colc = !p.sym && C.sn0 == 1 && !C.dst32;  // columns contiguous: stores go through the transpose tile
     const bool flip = !p.ws && p.asign < 0;
     const int ash = p.ws ? 0 : p.ashift;
     const bool mul = !p.ws && p.asign == 0;
@@ -364,92 +401,105 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
       }
       ++it;
       tc_fence_after();
-      const int m = ti.m0 + quad * 32 + lane, nbase = ti.n0 + part * kEpiCols;
-      const bool mok = m < ti.M;
-      const int ch = ti.kb0 / (kChunk / kBK);
-      const int ea = mok ? p.ea[static_cast<long long>(ch) * p.ea_rows + ti.a0 + m] : 0;
+      const int ch = ti.kb0 / (kChunk / kBK), kcol = ti.nkb * kBK;
       const long long cb = ti.cbase + (p.ws ? static_cast<long long>(ti.z) * p.M * p.N : 0);
-      const long long moff = mok ? out_moff(C, mb + m) : 0;
-      long long roff[4];  // destination rows of the transposed stores
-      if (colc) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int mm = ti.m0 + quad * 32 + 8 * q + lane / 4;
-          roff[q] = mm < ti.M ? cb + out_moff(C, mb + mm) : -1;
+      const float thr = 0x1p-9f * sqrtf(static_cast<float>(kcol));
+      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+      auto put = [&](long long off, double x) {
+        if (C.dst32) {
+          float y = static_cast<float>(x);
+          if (C.beta != 0.0) y += static_cast<float>(C.beta) * C.dst32[off];
+          C.dst32[off] = y;
+        } else if (C.beta == 0.0) {
+          C.dst[off] = x;
+        } else if (C.beta == 1.0) {
+          asm volatile("red.global.add.f64 [%0], %1;" ::"l"(C.dst + off), "d"(x) : "memory");
+        } else {
+          C.dst[off] = x + C.beta * C.dst[off];
         }
-      }
-      const uint32_t acc = tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * kEpiCols;
-#pragma unroll 1
-      for (int c4 = 0; c4 < kEpiCols / 4; ++c4) {
-        float v[8][4];
+      };
+      // unit: rows [16 half, + 16) of the quadrant, columns [8 grp, + 8) of the tile; a lane has rows m, m + 8 and
+      // columns n, n + 1 of it, na and nb2 of them inside
+      int m, n, na, nb2;
+      auto unit_at = [&](int x) {
+        const int unit = part + x * (kEpiWarps / 4);
+        m = ti.m0 + quad * 32 + 16 * (unit & 1) + lane / 4;
+        n = ti.n0 + 8 * (unit >> 1) + 2 * (lane & 3);
+        na = m + 8 < ti.M ? 2 : m < ti.M ? 1 : 0;
+        nb2 = n + 1 < p.N ? 2 : n < p.N ? 1 : 0;
+      };
+      auto store = [&](const double (&r)[4], unsigned which) {
+        long long moff[2], noff[2];
 #pragma unroll
-        for (int g = 0; g < 8; ++g) tmem_ld4(acc + g * kBN + 4 * c4, v[g]);
+        for (int h = 0; h < 2; ++h) {
+          moff[h] = h < na ? cb + out_moff(C, mb + m + 8 * h) : 0;
+          noff[h] = h < nb2 ? out_noff(C, nb + n + h) : 0;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int mm = mb + m + 8 * (e >> 1), nn = nb + n + (e & 1);
+          if (!(which >> e & 1u) || (e >> 1) >= na || (e & 1) >= nb2 || (p.sym && nn < mm)) continue;
+          put(moff[e >> 1] + noff[e & 1], r[e]);
+          if (p.sym && nn > mm) put(cb + out_moff(C, nn) + out_noff(C, mm), r[e]);
+        }
+      };
+      unsigned todo = 0;  // four bits per unit: elements to be summed in FP64
+#pragma unroll 1
+      for (int x = 0; x < kEpiUnits; ++x) {
+        const int unit = part + x * (kEpiWarps / 4);
+        float v[kSlices + 1][4];
+#pragma unroll
+        for (int g = 0; g <= kSlices; ++g)
+          tmem_ld_16x8(acc + (static_cast<uint32_t>(16 * (unit & 1)) << 16) + g * kBN + 8 * (unit >> 1), v[g]);
         tmem_wait_ld(v);
-        if (c4 == kEpiCols / 4 - 1) {  // everything read: the next tile's products may start
+        if (x == kEpiUnits - 1) {  // everything read: the next tile's products may start
           tc_fence_before();
           mbar_arrive(acce);
         }
-        const int n0 = nbase + 4 * c4;
-        if (n0 >= p.N || ti.m0 + quad * 32 >= ti.M) continue;  // nothing of this warp's is inside
+        if (ti.m0 + quad * 32 + 16 * (unit & 1) >= ti.M || ti.n0 + 8 * (unit >> 1) >= p.N) continue;  // nothing inside
+        unit_at(x);
+        int ea[2], eb[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          ea[h] = h < na ? p.ea[static_cast<long long>(ch) * p.ea_rows + ti.a0 + m + 8 * h] : 0;
+          eb[h] = h < nb2 ? p.eb[static_cast<long long>(ch) * p.eb_rows + ti.b0 + n + h] : 0;
+        }
         double r[4];
-        // lane j < 4 holds the exponent of column n0 + j
-        const int nl = n0 + (lane & 3);
-        const int ebl = nl < p.N ? p.eb[static_cast<long long>(ch) * p.eb_rows + ti.b0 + nl] : 0;
+        unsigned bad = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int n = n0 + j;
-          const int eb = __shfl_sync(0xffffffffu, ebl, j);
-          float a[8];
+        for (int e = 0; e < 4; ++e) {  // row e / 2, column e % 2
+          float a[kSlices];
 #pragma unroll
-          for (int g = 0; g < 8; ++g) a[g] = v[g][j];
+          for (int g = 0; g < kSlices; ++g) a[g] = v[g][e];
           long long hi;
           int lo;
           sl_combine(a, hi, lo);
-          if (ea == kBadExp || eb == kBadExp) {
-            r[j] = 0.0;
-            if (mok && n < p.N) {
-              const double x = sl_dot64(p.A64 + (ti.a0 + m) * p.lda, p.B64 + (ti.b0 + n) * p.ldb, ti.kb0 * kBK,
-                                        (ti.kb0 + ti.nkb) * kBK);
-              r[j] = p.ws ? x : C.alpha * x;
-            }
-          } else {
-            r[j] = sl_round(hi, lo, ea + eb + ash, flip);
-            if (mul) r[j] *= C.alpha;
-          }
+          const int xa = ea[e >> 1], xb = eb[e & 1];
+          const float T = v[kSlices][e];
+          const bool f = xa == kBadExp || xb == kBadExp || (T > 0.f && T < thr);
+          bad |= f ? 1u << e : 0u;
+          r[e] = sl_round(hi, lo, f ? 0 : xa + xb + ash, flip);
+          if (mul) r[e] *= C.alpha;
         }
-        auto put = [&](long long off, double x) {
-          if (C.dst32) {
-            float y = static_cast<float>(x);
-            if (C.beta != 0.0) y += static_cast<float>(C.beta) * C.dst32[off];
-            C.dst32[off] = y;
-          } else if (C.beta == 0.0) {
-            C.dst[off] = x;
-          } else if (C.beta == 1.0) {
-            asm volatile("red.global.add.f64 [%0], %1;" ::"l"(C.dst + off), "d"(x) : "memory");
-          } else {
-            C.dst[off] = x + C.beta * C.dst[off];
-          }
-        };
-        if (colc) {
-          __syncwarp();
+        store(r, ~bad);
+        if (na < 2) bad &= na == 0 ? 0u : 3u;
+        if (nb2 < 2) bad &= nb2 == 0 ? 0u : 5u;
+        todo |= bad << (4 * x);
+      }
+      if (__any_sync(0xffffffffu, todo != 0u)) {
+#pragma unroll 1
+        for (int x = 0; x < kEpiUnits; ++x) {
+          const unsigned need = todo >> (4 * x) & 15u;
+          if (!__any_sync(0xffffffffu, need != 0u)) continue;
+          unit_at(x);
+          double d[4] = {0.0, 0.0, 0.0, 0.0};
+          sl_dot64(p.A64 + (ti.a0 + m) * p.lda + ti.kb0 * kBK, 8 * p.lda, p.B64 + (ti.b0 + n) * p.ldb + ti.kb0 * kBK, p.ldb, kcol,
+                   need, d);
+          if (!p.ws) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) tile[lane * 5 + j] = r[j];
-          __syncwarp();
-          const int n = n0 + (lane & 3);
-          if (n < p.N) {
-            const long long noff = out_noff(C, nb + n);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (roff[q] >= 0) put(roff[q] + noff, tile[(8 * q + lane / 4) * 5 + (lane & 3)]);
+            for (int e = 0; e < 4; ++e) d[e] *= C.alpha;
           }
-        } else if (mok) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int n = n0 + j;
-            if (n >= p.N || (p.sym && nb + n < mb + m)) continue;
-            put(cb + moff + out_noff(C, nb + n), r[j]);
-            if (p.sym && nb + n > mb + m) put(cb + out_moff(C, nb + n) + out_noff(C, mb + m), r[j]);
-          }
+          store(d, need);
         }
       }
     }
@@ -460,9 +510,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_sl(const __grid_constant__
 }
 
 bool make_slice_map(CUtensorMap* map, const void* p, long long rows, int Kp, int box_rows) {
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(Kp), static_cast<cuuint64_t>(rows), kSlices};
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(Kp), static_cast<cuuint64_t>(rows), kPlanes};
   cuuint64_t strides[2] = {static_cast<cuuint64_t>(Kp) * 2, static_cast<cuuint64_t>(Kp) * 2 * static_cast<cuuint64_t>(rows)};
-  cuuint32_t box[3] = {kBK, static_cast<cuuint32_t>(box_rows), kSlices};
+  cuuint32_t box[3] = {kBK, static_cast<cuuint32_t>(box_rows), kPlanes};
   return encode_tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(p), dims, strides, box,
                            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
@@ -501,7 +551,7 @@ Sliced slice_at(void* mem, long long rows, int Kp, const double* src, long long 
   s.Kp = Kp;
   s.p = mem;
   s.ex = reinterpret_cast<int*>(static_cast<unsigned char*>(mem) +
-                                (static_cast<size_t>(rows) * Kp * 2 * kSlices + 255) / 256 * 256);
+                                (static_cast<size_t>(rows) * Kp * 2 * kPlanes + 255) / 256 * 256);
   s.src = src;
   s.ld = ld;
   return s;

@@ -7,8 +7,8 @@
 
 namespace lnocc {
 
-// Rows of a packed FP64 operand (row stride ld, Kp columns) as eight BF16 planes [8][rows][Kp] and the
-// exponents [ceil(Kp / 512)][rows] of their chunks.
+// Rows of a packed FP64 operand (row stride ld, Kp columns) as ten BF16 planes [10][rows][Kp] (nine digits and the
+// magnitudes) and the exponents [ceil(Kp / 512)][rows] of their chunks.
 struct Sliced {
   void* p = nullptr;
   int* ex = nullptr;

@@ -155,9 +155,9 @@ struct SplitWs {
 };
 SplitWs& split_ws();
 // Bytes of a slice workspace for products whose operands take at most `operand_bytes` packed in FP64: room
-// for the planes of both (16 bytes an element) up to 256 MB (panels beyond that).
+// for the planes of both (20 bytes an element) up to 256 MB (panels beyond that).
 inline size_t slice_ws_bytes(size_t operand_bytes) {
-  const size_t want = 4 * operand_bytes + (size_t(1) << 20);
+  const size_t want = 5 * operand_bytes + (size_t(1) << 20);
   return want < (size_t(256) << 20) ? want : size_t(256) << 20;
 }
 // Fixed-order sum of split-K partials (split_ws().p) into C, output rows / columns from m0 / n0.

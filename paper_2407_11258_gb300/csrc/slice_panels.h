@@ -6,11 +6,12 @@
 namespace lnocc {
 
 constexpr int kSliceChunk = 512;  // columns that share one exponent
-constexpr int kSlices = 8;        // BF16 digit planes of an operand
+constexpr int kSlices = 9;        // BF16 digit planes of an operand
+constexpr int kPlanes = 10;       // and the plane of its magnitudes
 
 // Device bytes of the planes and chunk exponents of `rows` rows of Kp columns.
 inline size_t slice_bytes(long long rows, int Kp) {
-  const size_t planes = static_cast<size_t>(rows) * Kp * 2 * kSlices;
+  const size_t planes = static_cast<size_t>(rows) * Kp * 2 * kPlanes;
   const size_t ex = static_cast<size_t>(rows) * ((Kp + kSliceChunk - 1) / kSliceChunk) * 4;
   return (planes + 255) / 256 * 256 + (ex + 255) / 256 * 256;
 }
