@@ -178,7 +178,7 @@ int lnocc_fragment_energy(lnocc_frag* f, int nlo, const double* U_frag, double* 
  *   e_t_full (host)         : canonical (T) energy, the trace of the (T) pair matrix (full active space).
  *   e_t_frag (host)         : sum_alpha sum_ii' U_i,alpha E_ii',(T) U_i',alpha (may be NULL).
  * FP64 precision: FP64 contractions and energy arithmetic (the digit planes of the contractions' operands,
- * up to 32 GB, are part of the temporaries). Mixed precision: the W contractions as
+ * up to 32 GB, are temporaries too where they fit; the call is slower without them). Mixed precision: the W contractions as
  * BF16x3/FP32 on tensor cores; the denominators' terms formed in FP64, the scaled w and v, their
  * products and the i-sums in FP32; a block's partials summed in compensated FP32 (the rounding error
  * of every addition carried alongside, both converted to FP64 once per block) by the staged kernels,
@@ -187,7 +187,7 @@ int lnocc_fragment_energy(lnocc_frag* f, int nlo, const double* U_frag, double* 
  * staged energy kernels run; otherwise a generic kernel that stages nothing).
  * Temporaries (the packed (T) operands, a W chunk of at most opts.triples_chunk_mb or one b-slab, the
  * per-block partial sums, the launch tables and the padded U) come from the attached workspace
- * (lnocc_frag_set_workspace; LNOCC_EINVAL if it is smaller than lnocc_workspace_bytes), or else are
+ * (lnocc_frag_set_workspace; LNOCC_EINVAL if it is too small), or else are
  * allocated in the fragment's memory mode and freed before the call returns (LNOCC_ENOMEM when they do
  * not fit). Synchronizes `stream`.
  */
@@ -215,13 +215,14 @@ int lnocc_triples_device(lnocc_frag* f, int nlo, const double* U_frag, double* e
 /*
  * lnocc_workspace_bytes -- device scratch that lnocc_triples needs for a fragment of these sizes
  * (Sec. II.D's (T) step: packed W/V operands, the W chunk and the block partial sums), for the precision
- * and opts->triples_chunk_mb of `opts` (NULL: defaults). *bytes receives the size.
+ * and opts->triples_chunk_mb of `opts` (NULL: defaults). *bytes receives the size. In FP64 precision it
+ * includes the digit planes of the operands; a workspace without room for them is accepted too.
  */
 int lnocc_workspace_bytes(int nocc, int nvir, int naux, const lnocc_opts* opts, long long* bytes);
 
 /*
- * lnocc_frag_set_workspace -- attach caller-owned device memory (at least lnocc_workspace_bytes bytes for
- * the fragment's sizes and options, else LNOCC_EINVAL) from which lnocc_triples takes its temporaries, so
+ * lnocc_frag_set_workspace -- attach caller-owned device memory (lnocc_workspace_bytes bytes for the fragment's
+ * sizes and options; LNOCC_EINVAL if it is smaller than lnocc_triples can work with) from which lnocc_triples takes its temporaries, so
  * that no call after lnocc_build_ints allocates. The caller keeps ownership; the memory must stay valid
  * while attached and must not be used by other work during lnocc_triples. NULL detaches.
  */

@@ -74,7 +74,7 @@ long long estimate_fragment_bytes(int o_, int v_, int N_, bool mixed, int n_refi
   };
   b += consts(mixed ? 4 : 8);
   if (mixed && n_refine > 0) b += consts(8);
-  if (do_t) b += static_cast<long long>(triples_plan(o_, v_, N_, mixed, chunk_mb).total);
+  if (do_t) b += static_cast<long long>(triples_plan(o_, v_, N_, mixed, chunk_mb, 0).alloc);
   return b + b / 16 + (64LL << 20);
 }
 

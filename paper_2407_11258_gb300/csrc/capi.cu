@@ -197,7 +197,7 @@ int lnocc_workspace_bytes(int nocc, int nvir, int naux, const lnocc_opts* opts, 
     return LNOCC_EINVAL;
   }
   *bytes = static_cast<long long>(
-      lnocc::triples_plan(nocc, nvir, naux, o.precision == LNOCC_PREC_MIXED, o.triples_chunk_mb).total);
+      lnocc::triples_plan(nocc, nvir, naux, o.precision == LNOCC_PREC_MIXED, o.triples_chunk_mb, 0).total);
   return LNOCC_OK;
 }
 
@@ -209,9 +209,9 @@ int lnocc_frag_set_workspace(lnocc_frag* h, void* workspace, long long workspace
   }
   Frag& f = h->f;
   if (workspace) {
-    const size_t need = lnocc::triples_plan(f.o, f.v, f.N, f.mixed, f.opts.triples_chunk_mb).total;
+    const size_t need = lnocc::triples_plan(f.o, f.v, f.N, f.mixed, f.opts.triples_chunk_mb, 0).need;
     if (workspace_bytes < 0 || static_cast<size_t>(workspace_bytes) < need) {
-      lnocc::set_error("lnocc_frag_set_workspace: workspace smaller than lnocc_workspace_bytes (" +
+      lnocc::set_error("lnocc_frag_set_workspace: workspace smaller than lnocc_workspace_bytes (at least " +
                        std::to_string(need) + " bytes)");
       return LNOCC_EINVAL;
     }

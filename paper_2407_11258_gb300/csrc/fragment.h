@@ -31,11 +31,17 @@ struct Consts {
 
 // Sizes (bytes) of the device temporaries of one lnocc_triples call (triples.cu).
 struct TriplesPlan {
-  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, tri, slxt, slto, total;
+  size_t xt, to, ovoo, pbvv, ovvv_chunk, w, tpart, batch, u, ovt, tri, slxt, slto;
+  size_t total;   // what lnocc_workspace_bytes reports
+  size_t need;    // the least attached workspace that is accepted
+  size_t alloc;   // what a call without an attached workspace allocates
+  size_t w_over;  // attached workspace, mixed: bytes by which W starts inside the B_vv and (jb|ad) temporaries
+  bool tri_over;  // attached workspace, mixed: the triple table lies in them
   long long welems, nblk;
   int bc, jp;
 };
-TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb);
+// avail: bytes of the attached workspace (0: none, the call allocates).
+TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avail);
 // Elements (FP64-sized) of each of the two packing scratch buffers of a fragment (ccsd.cu).
 long long packing_scratch_elems(int o, int v, int N);
 

@@ -466,11 +466,23 @@ __global__ void k_swap_outer_rows(const uint4* __restrict__ src, uint4* __restri
 // Device temporaries of one lnocc_triples call, in allocation order. Every size here is what the call
 // asks for; with a caller workspace attached the call carves them from it in this order (256-byte
 // aligned), so lnocc_workspace_bytes and the call agree by construction.
-TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
+//
+// What makes the call faster but can be done without never decides whether a workspace is large enough:
+//   * mixed: rows of W padded to 16 bytes, and the table of occupied triples. In an attached workspace W starts
+//     early by what the padding adds, inside the temporaries of the operands' assembly, which are no longer
+//     read when the first W is written, and the table lies at their start. Where those are too small for that
+//     (nvir below about nocc) and the workspace has no room, W is unpadded, the contractions run one per
+//     term and the energies in the generic kernel.
+//   * FP64: the digit planes of the four operands, cut once per call instead of in every product that reads them.
+//     An attached workspace without room for them, or a call whose allocations fail, runs without: sigma3, 4
+//     and 6 then cut their operands for every chunk into the handle's slice workspace, and the batched
+//     sigma1, 2 and 5 run on the SIMT kernel. The planes are left out beyond 32 GB (nocc 24 with nvir above 296).
+TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avail) {
   TriplesPlan p{};
   const long long oo = 1LL * o * o, vv = 1LL * v * v, ooo = oo * o;
   const size_t esz = bf ? 4 : 8;
   auto packed = [&](long long rows, int K) { return static_cast<size_t>(rows) * round_up(std::max(K, 1), 64) * esz; };
+  auto al = [](size_t x) { return (std::max<size_t>(x, 256) + 255) / 256 * 256; };
   const int Kt = v + o;
   p.xt = packed(vv * o, Kt);
   p.to = packed(v * oo, Kt);
@@ -478,35 +490,51 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb) {
   p.pbvv = packed(vv, N);
   p.bc = static_cast<int>(std::max(1LL, std::min<long long>(v, (1LL << 26) / (o * vv))));
   p.ovvv_chunk = static_cast<size_t>(p.bc) * o * vv * 8;
-  // W chunk: up to chunk_mb (fewer, larger contraction launches measured faster than chunks that fit
-  // L2), but never more than the largest slab (b + 1)(v - b) o^3 needs, and at least one c of a slab
-  p.jp = bf ? round_up(o, 4) : o;  // row length of W: 16-byte rows for the copies of the mixed path
-  const long long ooj = oo * p.jp;
-  long long max_slab = 0;
-  for (int bb = 0; bb < v; ++bb) max_slab = std::max(max_slab, 1LL * (bb + 1) * (v - bb) * ooj);
-  const long long cmb = chunk_mb > 0 ? chunk_mb : 768;
-  p.welems = std::max<long long>(std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab), v * ooj);
-  p.w = static_cast<size_t>(p.welems) * esz;
   p.nblk = 0;
   for (int b = 0; b < v; ++b) p.nblk += 1LL * (b + 1) * (v - b);
   p.tpart = static_cast<size_t>(p.nblk + 256) * 2 * 8;  // block partials, then 256 first-pass sums
   p.batch = sizeof(BatchEntry) * static_cast<size_t>(std::max(1LL, vv / 2 + v));  // one entry per (b, c >= b)
   p.u = static_cast<size_t>(o) * 8 * 8;  // U padded to at most 8 LOs
-  p.tri = static_cast<size_t>(tri_count(std::min(o, kMaxStagedOcc))) * 4;  // unordered occupied triples
   p.ovt = bf ? static_cast<size_t>(vv * oo) * 4 : 0;  // FP32 (ia|jb) in block-energy order (mixed)
-  auto al = [](size_t x) { return (std::max<size_t>(x, 256) + 255) / 256 * 256; };
-  // FP64: the digit planes of the four operands, cut once per call instead of in every product that reads
-  // them; beyond 32 GB (nocc 24 with nvir above 270) the products run on the SIMT kernel from the packed
-  // operands alone
-  const int Ktp = round_up(Kt, 64);
-  const size_t slxt = slice_bytes(vv * o, Ktp), slto = slice_bytes(v * oo, Ktp);
-  if (!bf && 2 * (slxt + slto) <= (size_t(32) << 30)) {
-    p.slxt = slxt;
-    p.slto = slto;
-    p.total += 2 * al(p.slxt) + 2 * al(p.slto);
+  // W chunk: up to chunk_mb (fewer, larger contraction launches measured faster than chunks that fit
+  // L2), but never more than the largest slab (b + 1)(v - b) o^2 jp needs, and at least one c of a slab
+  long long max_slab = 0;
+  for (int bb = 0; bb < v; ++bb) max_slab = std::max(max_slab, 1LL * (bb + 1) * (v - bb));
+  const long long cmb = chunk_mb > 0 ? chunk_mb : 768;
+  auto set_rows = [&](int jp) {  // rows of W of jp elements
+    p.jp = jp;
+    p.welems = std::max<long long>(std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab * oo * jp), v * oo * jp);
+    p.w = static_cast<size_t>(p.welems) * esz;
+  };
+  set_rows(o);
+  const size_t fixed = 2 * al(p.xt) + 2 * al(p.to) + al(p.ovoo) + al(p.pbvv) + al(p.ovvv_chunk) + al(p.tpart) +
+                       2 * al(p.batch) + al(p.u) + (bf ? al(p.ovt) : 0);
+  const size_t w_plain = al(p.w);
+  p.need = fixed + w_plain;
+  if (bf) {
+    p.tri = static_cast<size_t>(tri_count(std::min(o, kMaxStagedOcc))) * 4;
+    set_rows(round_up(o, 4));  // 16-byte rows for the copies
+    p.alloc = fixed + al(p.w) + al(p.tri);
+    const size_t over = al(p.w) - w_plain;
+    const bool fits = al(p.tri) + over <= al(p.pbvv) + al(p.ovvv_chunk);
+    p.total = fits ? p.need : p.alloc;
+    if (avail > 0 && fits) {
+      p.w_over = over;
+      p.tri_over = true;
+    } else if (avail > 0 && avail < p.total) {
+      set_rows(o);
+      p.tri = 0;
+    }
+  } else {
+    const int Ktp = round_up(Kt, 64);
+    const size_t slxt = slice_bytes(vv * o, Ktp), slto = slice_bytes(v * oo, Ktp), planes = 2 * al(slxt) + 2 * al(slto);
+    p.total = p.need + (planes <= (size_t(32) << 30) ? planes : 0);
+    p.alloc = p.total;
+    if (p.total > p.need && (avail == 0 || avail >= p.total)) {
+      p.slxt = slxt;
+      p.slto = slto;
+    }
   }
-  p.total += 2 * al(p.xt) + 2 * al(p.to) + al(p.ovoo) + al(p.pbvv) + al(p.ovvv_chunk) + al(p.w) + al(p.tpart) +
-            2 * al(p.batch) + al(p.u) + (bf ? al(p.ovt) + al(p.tri) : 0);
   return p;
 }
 
@@ -517,9 +545,9 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   // tile timing), so that the call can be captured into a CUDA graph; the energies and the device
   // status word are copied to the caller's device memory at the end of the stream's work
   const bool dev_out = e_dev != nullptr;
-  const TriplesPlan tp = triples_plan(o, v, N, bf, opts.triples_chunk_mb);
-  if (ws_ext && ws_ext_bytes < tp.total) {
-    set_error("lnocc_triples: attached workspace smaller than lnocc_workspace_bytes (" + std::to_string(tp.total) +
+  const TriplesPlan tp = triples_plan(o, v, N, bf, opts.triples_chunk_mb, ws_ext ? ws_ext_bytes : 0);
+  if (ws_ext && ws_ext_bytes < tp.need) {
+    set_error("lnocc_triples: attached workspace smaller than lnocc_workspace_bytes (at least " + std::to_string(tp.need) +
               " bytes)");
     return LNOCC_EINVAL;
   }
@@ -605,8 +633,10 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   pack_cols(view(ovoo, A_(v, oo), A_(o, v * oo), A_(o, o), kOne, kOne, A_(o, 1)), TO, 0, v, wl, s);
   pack_cols(view(ovoo, A_(v, oo), A_(o, o), A_(o, v * oo), kOne, kOne, A_(o, 1)), TOT, 0, v, wl, s);
   // (jb|ad) -> XT2[b][a][j][d], in chunks of b; XT1[y][a][i][d] = (ai|yd) = XT2[a][y][i][d]
+  void* dead = nullptr;  // start of the B_vv and (jb|ad) temporaries: free for others after this block
   {
     Packed PBvv = mk(static_cast<int>(vv), N);
+    dead = PBvv.p;
     if (!PBvv.p) {
       cleanup();
       set_error("lnocc_triples: device allocation failed (B_vv)");
@@ -647,7 +677,13 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   const int jp = tp.jp;
   const long long ooj = oo * jp;  // W elements of one (c, a)
   const long long welems = tp.welems;
-  void* W = tmp_alloc(tp.w);
+  void* W = nullptr;
+  if (ws_ext && tp.w_over > 0) {
+    W = static_cast<unsigned char*>(ws_ext) + ws_used - tp.w_over;
+    ws_used += (std::max<size_t>(tp.w, 256) + 255) / 256 * 256 - tp.w_over;
+  } else {
+    W = tmp_alloc(tp.w);
+  }
   const long long nblk_total = tp.nblk;
   double* tpart = static_cast<double*>(tmp_alloc(tp.tpart));
   // chunk plan and the per-c batch tables of the sigma2 / sigma5 terms (uploaded once)
@@ -692,7 +728,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   const long long small_smem = (3LL * o * (o + 1) + 4LL * o + 16LL * o + 4) * wsz;
   const bool staged_full = 2LL * sblk * wsz + small_smem <= 200LL * 1024;
   const bool staged =
-      (bf ? o <= kMaxStagedOcc : staged_full || sblk * wsz + small_smem <= 200LL * 1024) && nlo <= 8;
+      (bf ? o <= kMaxStagedOcc && tp.tri > 0 : staged_full || sblk * wsz + small_smem <= 200LL * 1024) && nlo <= 8;
   // the FP64 kernel is compiled for 0, 1, 2, 4 or 8 LOs: U zero-padded to the next size
   const int nlo_t = bf || nlo == 0 ? nlo : nlo <= 1 ? 1 : nlo <= 2 ? 2 : nlo <= 4 ? 4 : 8;
   const size_t esmem = (staged_full ? 2 : 1) * sblk * wsz + static_cast<size_t>(small_smem);  // FP64 kernel
@@ -711,7 +747,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   unsigned* tri = nullptr;
   if (bf && staged) {
     ovT = static_cast<float*>(tmp_alloc(tp.ovt));
-    tri = static_cast<unsigned*>(tmp_alloc(tp.tri));
+    tri = static_cast<unsigned*>(ws_ext && tp.tri_over ? dead : tmp_alloc(tp.tri));
     if (!ovT || !tri) {
       cleanup();
       set_error("lnocc_triples: device allocation failed (ovT)");
@@ -723,7 +759,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   }
   Sliced sls[4];
   if (tp.slxt > 0) {
-    // allocated last: without room for the planes the products run on the SIMT kernel from the packed operands
+    // allocated last: the call runs without them if they do not fit (triples_plan)
     Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
     void* mem[4];
     const size_t n_mine = mine.size();
@@ -802,7 +838,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   const long long oj = 1LL * o * jp;  // W strides: a ooj, i oj, k jp, j 1
   // grouped launches (two per chunk instead of five): nocc 16 and 32, where 128-row tiles hold whole a values
   // and a (y, z) plane is one or four 256-column tiles, in gemm.cu; any other nocc from 4 to 32 in triples_gemm.cu
-  const bool grouped = bf && o >= 4 && o <= 32 && opts.triples_kernel != LNOCC_TK_PER_TERM;
+  const bool grouped = bf && o >= 4 && o <= 32 && jp % 4 == 0 && opts.triples_kernel != LNOCC_TK_PER_TERM;
   const Packed* ops_k2[4] = {&TO, &XT2, &XT2, &XT1};
   const Packed* ops_a[4] = {&XT1, &TO, &XT2, &TOT};
   const Packed* ops_b[4] = {&TO, &XT2, &TO, &XT1};
