@@ -276,8 +276,9 @@ int lnocc_gemm_noalloc(int precision, int M, int N, int K, const double* A, cons
  *   nocc, nvir, naux   : the system's occupied, virtual and auxiliary dimensions (nocc * nvir <= 2^30).
  *   eps [nocc + nvir]  : canonical orbital energies (device), occupied first; every virtual above every occupied.
  *   B_ov [naux][nocc][nvir] : the occupied-virtual block of the DF factors (device).
- *   workspace, workspace_bytes : caller-owned device scratch of at least lnocc_mp2_workspace_bytes(...) bytes,
- *                        or NULL (the call then allocates and frees its own); LNOCC_EINVAL when too small.
+ *   workspace, workspace_bytes : caller-owned device scratch of lnocc_mp2_workspace_bytes(...) bytes, or NULL (the
+ *                        call then allocates and frees its own); LNOCC_EINVAL when too small. (For some large
+ *                        systems in FP64 the size includes up to 256 MB that the call can do without, slower.)
  *   e_mp2 (host)       : the energy (Eh).
  * The sum over blocks is taken in a fixed order (repeatable bit for bit). Synchronizes `stream`.
  */

@@ -574,8 +574,7 @@ void splitk_reduce(int splits, int M, int N, const OutMap& C, cudaStream_t s, in
 // pipe (two FMA lanes per clock and SM: 1.1 TFLOP/s over the chip, and 68 us for a single 64 x 64 tile with
 // K = 64 however small the problem).
 void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s, int* dstatus) {
-  if (gemm_f64_slices(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, K, A.Kp, C, false, 0, 0, s,
-                      dstatus))
+  if (gemm_f64_slices(static_cast<const double*>(A.p), static_cast<const double*>(B.p), M, N, K, A.Kp, C, false, s, dstatus))
     return;
   const long long tiles = static_cast<long long>((N + 63) / 64) * ((M + 63) / 64);
   const int nk16 = A.Kp / 16;
@@ -595,23 +594,10 @@ void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s, int* 
   st.launches++;
   st.flops += 1.0 * M * M * A.Kp;  // half of 2 M^2 K
   const double* a = static_cast<const double*>(A.p);
-  if (gemm_f64_slices(a, a, M, M, A.Kp, A.Kp, C, true, 0, 0, s, dstatus)) return;
+  if (gemm_f64_slices(a, a, M, M, A.Kp, A.Kp, C, true, s, dstatus)) return;
   dim3 grid((M + 63) / 64, (M + 63) / 64, 1);
   count_launch();
   k_gemm_f64<true><<<grid, 256, 0, s>>>(a, a, M, M, A.Kp, C, A.Kp, nullptr, nullptr, 0);
-}
-
-void gemm_f64_lower(const Packed& A, int a_row0, int M, int N, int block, const OutMap& C, cudaStream_t s, int* dstatus) {
-  if (M <= 0 || N <= 0) return;
-  GemmStats& st = gemm_stats();
-  const double* a = static_cast<const double*>(A.p);
-  const double* a0 = a + static_cast<size_t>(a_row0) * A.Kp;
-  st.launches++;
-  st.flops += 2.0 * M * N * A.Kp;
-  if (gemm_f64_slices(a0, a, M, N, A.Kp, A.Kp, C, false, block, a_row0, s, dstatus)) return;
-  Packed A0 = A, B0 = A;
-  A0.p = const_cast<double*>(a0);
-  gemm_f64(A0, B0, M, N, A.Kp, C, s, dstatus);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -636,9 +636,17 @@ void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dba
   gemm_sliced_rows(A, 0, B, 0, maxM, N, K, C, 0, 0, dbatch, nbatch, seg, 0, 0, 0, s, dstatus);
 }
 
+void gemm_sliced_lower(const Sliced& A, int a_row0, int M, int N, int K, int block, const OutMap& C, cudaStream_t s,
+                       int* dstatus) {
+  GemmStats& st = gemm_stats();
+  st.launches++;
+  st.flops += 2.0 * M * N * K;
+  gemm_sliced_rows(A, a_row0, A, 0, M, N, K, C, 0, 0, nullptr, 1, 0, 0, block, a_row0, s, dstatus);
+}
+
 // A (M rows) and B (N rows) packed FP64, K = Kp: slices panels of both into the slice workspace.
-bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym, int tri,
-                     int tri_row0, cudaStream_t s, int* dstatus) {
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym,
+                     cudaStream_t s, int* dstatus) {
   const SplitWs& w = split_ws();
   if (!w.sl || !dstatus) return false;
   unsigned char* base = static_cast<unsigned char*>(w.sl);
@@ -646,7 +654,7 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int 
   if (same && slice_bytes(M, Kp) <= w.sl_bytes) {
     const Sliced SA = slice_at(base, M, Kp, A, Kp);
     slice(SA, s);
-    gemm_sliced_rows(SA, 0, SA, 0, M, N, K, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+    gemm_sliced_rows(SA, 0, SA, 0, M, N, K, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, 0, 0, s, dstatus);
     return true;
   }
   const SlicePanels pl = plan_slice_panels(M, N, Kp, w.sl_bytes);
@@ -659,7 +667,7 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int 
     const Sliced SA = slice_at(base + slice_bytes(nn, kw), mm, kw, A + static_cast<size_t>(m0) * Kp + k0, Kp);
     launch_slice(SA, first ? &SB : nullptr, s);
     Ck.beta = k0 == 0 ? C.beta : 1.0;
-    gemm_sliced_rows(SA, 0, SB, 0, mm, nn, ku, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, tri, tri_row0, s, dstatus);
+    gemm_sliced_rows(SA, 0, SB, 0, mm, nn, ku, Ck, m0, n0, nullptr, 1, 0, sym ? 1 : 0, 0, 0, s, dstatus);
   });
   return true;
 }

@@ -23,10 +23,14 @@ void gemm_sliced(const Sliced& A, int a_row0, const Sliced& B, int b_row0, int M
                  cudaStream_t s, int* dstatus);
 void gemm_sliced_batched(const Sliced& A, const Sliced& B, const BatchEntry* dbatch, int nbatch, int maxM, int N, int K,
                          int seg, const OutMap& C, cudaStream_t s, int* dstatus);
+// Rows [a_row0, a_row0 + M) of A against rows [0, N) of A; only elements whose column block n / block does not exceed
+// the row block (a_row0 + m) / block are needed (others may be left unset).
+void gemm_sliced_lower(const Sliced& A, int a_row0, int M, int N, int K, int block, const OutMap& C, cudaStream_t s,
+                       int* dstatus);
 // C = A B^T for packed FP64 operands through the thread's slice workspace (split_ws().sl): false when
 // there is none (or it is too small): the caller then runs the FP64 SIMT kernel. sym: A == B, the upper
-// part computed and mirrored. tri > 0: only elements with n / tri <= (tri_row0 + m) / tri are needed.
-bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym, int tri,
-                     int tri_row0, cudaStream_t s, int* dstatus);
+// part computed and mirrored.
+bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int Kp, const OutMap& C, bool sym,
+                     cudaStream_t s, int* dstatus);
 
 }  // namespace lnocc

@@ -90,9 +90,6 @@ void permute(const View& v, double* dst, double beta, cudaStream_t s);
 void gemm_f64(const Packed& A, const Packed& B, int M, int N, int K, const OutMap& C, cudaStream_t s, int* dstatus);
 // C = A A^T in FP64 with the symmetric half computed once and mirrored (A FP64-packed, M rows)
 void gemm_f64_sym(const Packed& A, int M, const OutMap& C, cudaStream_t s, int* dstatus);
-// Rows [a_row0, a_row0 + M) of A against rows [0, N) of A in FP64; only elements whose column block
-// n / block does not exceed the row block (a_row0 + m) / block are needed (others may be left unset).
-void gemm_f64_lower(const Packed& A, int a_row0, int M, int N, int block, const OutMap& C, cudaStream_t s, int* dstatus);
 void gemm_tc(const Packed& A, int a_row0, const Packed& B, int b_row0, int M, int N, const OutMap& C,
              cudaStream_t s, int* dstatus);
 // rows [a_row0, a_row0 + M) of A against rows [b_row0, b_row0 + N) of B

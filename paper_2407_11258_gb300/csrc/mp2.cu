@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <string>
 
+#include "gemm_slices.h"
 #include "internal.h"
 
 namespace lnocc {
@@ -95,15 +96,25 @@ __global__ void k_mp2_sum(const double* __restrict__ part, long long n, double* 
 }
 
 struct Mp2Plan {
-  size_t status, packed, X, part, slices, total;
-  int ni;
+  size_t status, packed, X, part, slices, extra;
+  size_t total;  // what lnocc_mp2_workspace_bytes reports
+  size_t need;   // the least workspace that is accepted
+  int ni, kw;    // occupied rows of an X chunk; columns of a panel of digit planes inside it (0: none)
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-Mp2Plan mp2_plan(bool bf, int o, int v, int N) {
+// FP64: the digit planes of B_ov take their place from the X chunk, which gets shorter, so that the workspace is no
+// larger than the SIMT kernel needs. They are whole, cut once, or in up to four panels of K, cut again for
+// every chunk and added up in X: the number of panels with the fewest launches (small systems are bound by
+// those). Where X leaves too little for any of them, or so little that cutting would take as long as the products
+// (a chunk below 256 rows), large systems ask for up to 256 MB more, but run on the SIMT kernel when given no more
+// than they need; small ones (X below 32 MB) keep what fits, or stay on the SIMT kernel. (30, 200, 640) 2.1 ms
+// as with a workspace of their own; (12, 120, 400) 0.44 ms in two panels and two chunks, 0.54 ms with whole planes
+// and six chunks, 0.34 ms with a workspace of their own; on the SIMT kernel 38.7 and 2.1 ms.
+Mp2Plan mp2_plan(bool bf, int o, int v, int N, size_t avail) {  // avail: the caller's workspace, 0: none
   Mp2Plan p{};
-  const size_t Kp = static_cast<size_t>(round_up(N, 64));
+  const int Kp = round_up(N, 64);
   const size_t ov = static_cast<size_t>(o) * v;
   // X chunk: ni * v rows of o * v FP64 columns, at most 512 MB (at least one occupied row)
   const size_t row_bytes = ov * v * 8;
@@ -113,8 +124,29 @@ Mp2Plan mp2_plan(bool bf, int o, int v, int N) {
   p.packed = align256(ov * Kp * (bf ? 4 : 8));
   p.X = align256(static_cast<size_t>(p.ni) * row_bytes);
   p.part = align256(static_cast<size_t>(T) * (T + 1) / 2 * o * p.ni * 8 + 8);
-  p.slices = bf ? 0 : align256(slice_ws_bytes(p.packed / 2));  // digit planes of B_ov (up to 256 MB)
-  p.total = p.status + p.packed + p.X + p.part + p.slices;
+  p.need = p.total = p.status + p.packed + p.X + p.part;
+  if (bf) return p;
+  const size_t room = p.X;
+  const bool large = room >= (size_t(32) << 20);
+  int best = 0;
+  for (int panels = 1; panels <= 4; ++panels) {
+    const int kw = round_up((Kp + panels - 1) / panels, 64), np = (Kp + kw - 1) / kw;
+    const size_t planes = slice_bytes(static_cast<long long>(ov), kw);
+    if (planes + row_bytes > room) continue;
+    const int ni = static_cast<int>(std::min<size_t>(o, (room - planes) / row_bytes)), chunks = (o + ni - 1) / ni;
+    const int launches = np == 1 ? 1 + 3 * chunks : chunks * (2 + 2 * np);
+    if ((best != 0 && launches >= best) || (large && np > 1 && 1LL * ni * v < 256)) continue;
+    best = launches;
+    p.ni = ni;
+    p.kw = kw;
+    p.slices = planes;
+    p.X = room - planes;
+  }
+  if (best == 0 && large) {
+    const size_t more = align256(slice_ws_bytes(p.packed));
+    p.total += more;
+    if (avail == 0 || avail >= p.total) p.extra = more;
+  }
   return p;
 }
 
@@ -129,7 +161,7 @@ extern "C" int lnocc_mp2_workspace_bytes(int precision, int nocc, int nvir, int 
     set_error("lnocc_mp2_workspace_bytes: bad arguments");
     return LNOCC_EINVAL;
   }
-  *bytes = static_cast<long long>(mp2_plan(precision == LNOCC_PREC_MIXED, nocc, nvir, naux).total);
+  *bytes = static_cast<long long>(mp2_plan(precision == LNOCC_PREC_MIXED, nocc, nvir, naux, 0).total);
   return LNOCC_OK;
 }
 
@@ -144,14 +176,15 @@ extern "C" int lnocc_mp2_energy(int precision, int nocc, int nvir, int naux, con
     return LNOCC_EINVAL;
   }
   const bool bf = precision == LNOCC_PREC_MIXED;
-  const Mp2Plan plan = mp2_plan(bf, nocc, nvir, naux);
+  const Mp2Plan plan =
+      mp2_plan(bf, nocc, nvir, naux, workspace ? static_cast<size_t>(std::max(workspace_bytes, 0LL)) : 0);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   unsigned char* base = static_cast<unsigned char*>(workspace);
   bool own = false;
   if (base) {
-    if (workspace_bytes < static_cast<long long>(plan.total)) {
-      set_error("lnocc_mp2_energy: workspace smaller than lnocc_mp2_workspace_bytes (" +
-                std::to_string(plan.total) + " bytes)");
+    if (workspace_bytes < static_cast<long long>(plan.need)) {
+      set_error("lnocc_mp2_energy: workspace smaller than lnocc_mp2_workspace_bytes (at least " +
+                std::to_string(plan.need) + " bytes)");
       return LNOCC_EINVAL;
     }
   } else {
@@ -171,7 +204,7 @@ extern "C" int lnocc_mp2_energy(int precision, int nocc, int nvir, int naux, con
   PA.Kp = round_up(naux, 64);
   PA.p = base + plan.status;
   double* X = reinterpret_cast<double*>(base + plan.status + plan.packed);
-  double* part = reinterpret_cast<double*>(base + plan.status + plan.packed + plan.X);
+  double* part = reinterpret_cast<double*>(base + plan.need - plan.part);
   const int o = nocc, v = nvir, N = naux;
   const long long ov = 1LL * o * v;
   int st = LNOCC_OK;
@@ -181,18 +214,31 @@ extern "C" int lnocc_mp2_energy(int precision, int nocc, int nvir, int naux, con
     pack(view(B_ov, kOne, Ax{o, v}, Ax{v, 1}, kOne, kOne, Ax{N, ov}), PA, s);
     const SplitWs saved = split_ws();
     split_ws() = SplitWs{};  // no split-K: its partials would need workspace beyond the plan
-    if (plan.slices > 0) {
-      split_ws().sl = base + plan.status + plan.packed + plan.X + plan.part;
-      split_ws().sl_bytes = plan.slices;
+    if (plan.extra > 0) {
+      split_ws().sl = base + plan.need;
+      split_ws().sl_bytes = plan.extra;
     }
+    Sliced planes;
+    auto cut = [&](int rows, int k0) {
+      planes = slice_at(base + plan.status + plan.packed + plan.X, rows, std::min(plan.kw, PA.Kp - k0),
+                        static_cast<const double*>(PA.p) + k0, PA.Kp);
+      slice(planes, s);
+    };
+    if (plan.kw >= PA.Kp) cut(PA.rows, 0);  // whole: once for all chunks
     const int T = (v + kTile - 1) / kTile;
     for (int i0 = 0; i0 < o; i0 += plan.ni) {
       const int ni = std::min(plan.ni, o - i0);
       const int ncols = (i0 + ni) * v;  // pairs j <= i only
-      if (bf)
+      if (plan.kw == 0) {
         gemm_off(PA, i0 * v, PA, 0, ni * v, ncols, N, out_rowmajor(X, ncols), s, dstatus);
-      else  // pairs j > i are not read: their tiles are skipped
-        gemm_f64_lower(PA, i0 * v, ni * v, ncols, v, out_rowmajor(X, ncols), s, dstatus);
+      } else {
+        for (int k0 = 0; k0 < N; k0 += plan.kw) {
+          if (plan.kw < PA.Kp) cut(ncols, k0);
+          // pairs j > i are not read: their tiles are skipped
+          gemm_sliced_lower(planes, i0 * v, ni * v, ncols, std::min(plan.kw, N - k0), v,
+                            out_rowmajor(X, ncols, 1.0, k0 > 0 ? 1.0 : 0.0), s, dstatus);
+        }
+      }
       dim3 grid(T * (T + 1) / 2, i0 + ni, ni);
       count_launch(2);
       k_mp2_pairs<<<grid, 256, 0, s>>>(X, ncols, i0, ni, o, v, eps, part);
