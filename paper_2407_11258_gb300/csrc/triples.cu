@@ -718,8 +718,13 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     set_error("lnocc_triples: device allocation failed (W chunk)");
     return LNOCC_ENOMEM;
   }
-  count_launch();
-  k_batch_tables<<<(v + 127) / 128, 128, 0, s>>>(o, v, jp, welems, dbat, dbat12);
+  // grouped launches (two per chunk instead of five): nocc 16 and 32, where 128-row tiles hold whole a values
+  // and a (y, z) plane is one or four 256-column tiles, in gemm.cu; any other nocc from 4 to 32 in triples_gemm.cu
+  const bool grouped = bf && o >= 4 && o <= 32 && jp % 4 == 0 && opts.triples_kernel != LNOCC_TK_PER_TERM;
+  if (!grouped) {  // the tables serve the batched per-term launches
+    count_launch();
+    k_batch_tables<<<(v + 127) / 128, 128, 0, s>>>(o, v, jp, welems, dbat, dbat12);
+  }
 
   // Block energy kernel. Mixed: w and v staged side by side while they fit (nocc <= 28: 182 KB at 28), one
   // value per element up to nocc 37 (203 KB), at most 8 LOs; FP64: w and v or w alone within 200 KB.
@@ -836,9 +841,6 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   };
   const int o2 = static_cast<int>(oo);
   const long long oj = 1LL * o * jp;  // W strides: a ooj, i oj, k jp, j 1
-  // grouped launches (two per chunk instead of five): nocc 16 and 32, where 128-row tiles hold whole a values
-  // and a (y, z) plane is one or four 256-column tiles, in gemm.cu; any other nocc from 4 to 32 in triples_gemm.cu
-  const bool grouped = bf && o >= 4 && o <= 32 && jp % 4 == 0 && opts.triples_kernel != LNOCC_TK_PER_TERM;
   const Packed* ops_k2[4] = {&TO, &XT2, &XT2, &XT1};
   const Packed* ops_a[4] = {&XT1, &TO, &XT2, &TOT};
   const Packed* ops_b[4] = {&TO, &XT2, &TO, &XT1};
