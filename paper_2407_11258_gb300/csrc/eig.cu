@@ -4,8 +4,8 @@
 // m = n rounded up to even players: in round r, pair 0 is (m - 1, r) and pair k >= 1 is
 // ((r + k) mod (m - 1), (r - k) mod (m - 1)). The m / 2 pairs of one round are disjoint, so their plane
 // rotations commute: every A_pq of the round is zeroed at once, A <- J^T A J as independent 2 x 2 blocks (rows of
-// pair P, columns of pair Q) and V <- V J. One cooperative kernel runs a whole sweep with a grid barrier
-// between rounds (k_jac_sweep). A player
+// pair P, columns of pair Q) and V <- V J. Up to order kSweepMax one cooperative kernel runs a whole sweep with a
+// grid barrier between rounds (k_jac_sweep); above, a round is two launches (k_jac_angles, k_jac_rotate). A player
 // index >= n (odd n) is a bye. Rotation angles follow the classical form: theta = (A_qq - A_pp) / 2A_pq,
 // t = sgn(theta) / (|theta| + sqrt(theta^2 + 1)), c = 1 / sqrt(1 + t^2), s = t c, which gives
 // A'_pp = A_pp - t A_pq, A'_qq = A_qq + t A_pq, A'_pq = 0. After each sweep the off-diagonal norm is read
@@ -54,6 +54,59 @@ __device__ __forceinline__ double2 jac_angle(const double* A, int n, int m, int 
   return make_double2(c, s);
 }
 
+// The 2 x 2 block (a b; c d) of A under the rotations of its row pair and its column pair; diag: the pair itself,
+// whose off-diagonal element the rotation annihilates.
+__device__ __forceinline__ void jac_block(double& a, double& b, double& c, double& d, double2 g1, double2 g2, bool diag) {
+  // rows: p <- c row_p - s row_q, q <- s row_p + c row_q
+  const double a1 = g1.x * a - g1.y * c, b1 = g1.x * b - g1.y * d;
+  const double c1 = g1.y * a + g1.x * c, d1 = g1.y * b + g1.x * d;
+  // columns: p <- c col_p - s col_q, q <- s col_p + c col_q
+  a = g2.x * a1 - g2.y * b1;
+  b = diag ? 0.0 : g2.y * a1 + g2.x * b1;
+  c = diag ? 0.0 : g2.x * c1 - g2.y * d1;
+  d = g2.y * c1 + g2.x * d1;
+}
+
+// A round of a large matrix: all angles, then (m/2)^2 blocks of A and n * (m/2) row-pairs of V in place.
+__global__ void k_jac_angles(const double* __restrict__ A, int n, int m, int r, double2* __restrict__ cs) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < m / 2) cs[k] = jac_angle(A, n, m, r, k);
+}
+__global__ void k_jac_rotate(double* __restrict__ A, double* __restrict__ V, int n, int m, int r,
+                             const double2* __restrict__ cs) {
+  const long long h = m / 2, nA = h * h, nV = static_cast<long long>(n) * h;
+  for (long long w = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; w < nA + nV;
+       w += static_cast<long long>(gridDim.x) * blockDim.x) {
+    if (w < nA) {
+      const int kP = static_cast<int>(w / h), kQ = static_cast<int>(w % h);
+      int p1, q1, p2, q2;
+      jac_pair(r, kP, m, &p1, &q1);
+      jac_pair(r, kQ, m, &p2, &q2);
+      const bool r1 = p1 < n, r2 = q1 < n, c1 = p2 < n, c2 = q2 < n;  // byes are absent rows / columns
+      double* R1 = A + static_cast<long long>(p1) * n;
+      double* R2 = A + static_cast<long long>(q1) * n;
+      double a = (r1 && c1) ? R1[p2] : 0.0, b = (r1 && c2) ? R1[q2] : 0.0;
+      double c = (r2 && c1) ? R2[p2] : 0.0, d = (r2 && c2) ? R2[q2] : 0.0;
+      jac_block(a, b, c, d, cs[kP], cs[kQ], kP == kQ);
+      if (r1 && c1) R1[p2] = a;
+      if (r1 && c2) R1[q2] = b;
+      if (r2 && c1) R2[p2] = c;
+      if (r2 && c2) R2[q2] = d;
+    } else {
+      const long long x = w - nA;
+      const int k = static_cast<int>(x % h);
+      int p, q;
+      jac_pair(r, k, m, &p, &q);
+      if (p >= n || q >= n) continue;
+      const double2 g = cs[k];
+      double* row = V + (x / h) * n;
+      const double vp = row[p], vq = row[q];
+      row[p] = g.x * vp - g.y * vq;
+      row[q] = g.y * vp + g.x * vq;
+    }
+  }
+}
+
 // All blocks of the grid arrive and wait for each other (cooperative launch: all are resident). The wait has a
 // wall-clock budget; when it runs out the flag is set and every block returns.
 __device__ bool jac_barrier(unsigned* count, unsigned target, int* flag) {
@@ -86,7 +139,9 @@ __device__ bool jac_barrier(unsigned* count, unsigned target, int* flag) {
 // matrix. What others wrote in the round before is read past L1 (__ldcg). Bound by latency: a round is one
 // dependent chain (three elements from L2, a square root and two divisions in FP64, the barrier). With two
 // launches per round (angles, rotations) a round took 10 us; the 1471 rounds of three matrices of order 160, 100
-// and 16 and three small ones fell from 15 to 8.8 ms. (t = 2 a_pq / (|d| + sqrt(d^2 + 4 a_pq^2)) would shorten
+// and 16 and three small ones fell from 15 to 8.8 ms. lnocc_lno_select, sweep against two launches per round:
+// order 333 26.4 and 42.3 ms, 500 54 and 81, 1000 222 and 236, 2000 1485 and 1323 (the rotations bound, and in place
+// they keep a third less in L2). (t = 2 a_pq / (|d| + sqrt(d^2 + 4 a_pq^2)) would shorten
 // the chain, but the zero eigenvalues of rank-deficient LO sets then come out as rounding noise.)
 __global__ void __launch_bounds__(256) k_jac_sweep(double* A0, double* A1, double* V, int n, int m, int tP, int tQ,
                                                    int tV, unsigned* count, int* flag) {
@@ -107,23 +162,16 @@ __global__ void __launch_bounds__(256) k_jac_sweep(double* A0, double* A1, doubl
         int p1, q1, p2, q2;
         jac_pair(r, kP, m, &p1, &q1);
         jac_pair(r, kQ, m, &p2, &q2);
-        const double2 g1 = ang[w / nq], g2 = ang[np + w % nq];
         const bool r1 = p1 < n, r2 = q1 < n, c1 = p2 < n, c2 = q2 < n;  // byes are absent rows / columns
-        const double a = (r1 && c1) ? __ldcg(A + static_cast<long long>(p1) * n + p2) : 0.0;
-        const double b = (r1 && c2) ? __ldcg(A + static_cast<long long>(p1) * n + q2) : 0.0;
-        const double cc = (r2 && c1) ? __ldcg(A + static_cast<long long>(q1) * n + p2) : 0.0;
-        const double d = (r2 && c2) ? __ldcg(A + static_cast<long long>(q1) * n + q2) : 0.0;
-        // rows: p <- c row_p - s row_q, q <- s row_p + c row_q
-        const double a1 = g1.x * a - g1.y * cc, b1 = g1.x * b - g1.y * d;
-        const double c1v = g1.y * a + g1.x * cc, d1 = g1.y * b + g1.x * d;
-        // columns: p <- c col_p - s col_q, q <- s col_p + c col_q
-        double a2 = g2.x * a1 - g2.y * b1, b2 = g2.y * a1 + g2.x * b1;
-        double c2v = g2.x * c1v - g2.y * d1, d2 = g2.y * c1v + g2.x * d1;
-        if (kP == kQ) b2 = c2v = 0.0;  // the element this rotation annihilates
-        if (r1 && c1) B[static_cast<long long>(p1) * n + p2] = a2;
-        if (r1 && c2) B[static_cast<long long>(p1) * n + q2] = b2;
-        if (r2 && c1) B[static_cast<long long>(q1) * n + p2] = c2v;
-        if (r2 && c2) B[static_cast<long long>(q1) * n + q2] = d2;
+        double a = (r1 && c1) ? __ldcg(A + static_cast<long long>(p1) * n + p2) : 0.0;
+        double b = (r1 && c2) ? __ldcg(A + static_cast<long long>(p1) * n + q2) : 0.0;
+        double c = (r2 && c1) ? __ldcg(A + static_cast<long long>(q1) * n + p2) : 0.0;
+        double d = (r2 && c2) ? __ldcg(A + static_cast<long long>(q1) * n + q2) : 0.0;
+        jac_block(a, b, c, d, ang[w / nq], ang[np + w % nq], kP == kQ);
+        if (r1 && c1) B[static_cast<long long>(p1) * n + p2] = a;
+        if (r1 && c2) B[static_cast<long long>(p1) * n + q2] = b;
+        if (r2 && c1) B[static_cast<long long>(q1) * n + p2] = c;
+        if (r2 && c2) B[static_cast<long long>(q1) * n + q2] = d;
       } else {
         const int x = w - nA;
         int p, q;
@@ -237,8 +285,11 @@ int grid_of(long long work, int threads) {
 
 }  // namespace
 
-// Doubles of scratch that sym_eig needs: norms, barrier and flag, then the second copy of the matrix.
-size_t eig_scratch(int n) { return 16 + static_cast<size_t>(n) * n; }
+// Largest order whose sweeps run in one launch (both forms measured at k_jac_sweep).
+constexpr int kSweepMax = 1024;
+
+// Doubles of scratch that sym_eig needs: norms, barrier and flag, then the second copy of the matrix or the angles.
+size_t eig_scratch(int n) { return 16 + (n <= kSweepMax ? static_cast<size_t>(n) * n : static_cast<size_t>(n) + 1); }
 
 // A [n][n] symmetric (destroyed); on return w [n] holds the eigenvalues (decreasing when desc, else
 // increasing), order [n] their columns in V, and V [n][n] the eigenvectors as columns (A V = V diag).
@@ -260,10 +311,12 @@ int sym_eig(double* A, double* V, double* w, int* order, int n, bool desc, doubl
   int sweep = 0;
   double hn[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if (n > 1) {
-    // about one 2 x 2 block or row pair a thread, at most one block per SM (all resident); a grid of tiles
-    // close to square keeps the angles each block needs few
+    // about one 2 x 2 block or row pair a thread, in one block per SM or, for larger orders, three (768 threads of
+    // 32 registers: all resident): order 333 26.4 and 26.6 ms with one and three, 500 61 and 54, 1000 299 and
+    // 222 (256 with eight: the barrier). A grid of tiles close to square keeps the angles each block needs few.
     const long long work = 1LL * h * h + 1LL * n * h;
-    const int blocks = static_cast<int>(std::max(1LL, std::min<long long>(num_sms(), (work + 255) / 256)));
+    const int cap = num_sms() * (n > 400 ? 3 : 1);
+    const int blocks = static_cast<int>(std::max(1LL, std::min<long long>(cap, (work + 255) / 256)));
     int gx = std::max(1, static_cast<int>(std::sqrt(static_cast<double>(blocks))));
     gx = std::min(gx, h);
     const int tP = (h + gx - 1) / gx;
@@ -286,6 +339,15 @@ int sym_eig(double* A, double* V, double* w, int* order, int n, bool desc, doubl
         return LNOCC_ENUMERIC;
       }
       if (hn[0] <= 1e-30 * hn[1] || hn[0] == 0.0) break;
+      if (n > kSweepMax) {
+        double2* cs = reinterpret_cast<double2*>(A2);
+        for (int r = 0; r < m - 1; ++r) {
+          count_launch(2);
+          k_jac_angles<<<grid_of(h, 128), 128, 0, s>>>(A, n, m, r, cs);
+          k_jac_rotate<<<grid_of(work, 256), 256, 0, s>>>(A, V, n, m, r, cs);
+        }
+        continue;
+      }
       LN_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned), s));
       void* args[] = {&A, &A2, &V, &nn, &mm, &tPa, &tQa, &tV, &count, &flag};
       count_launch();
