@@ -73,6 +73,7 @@ extern "C" {
 
 #define LNOCC_FAULT_NAN_INPUT 1 /* fault injection (host side): poison one element of the B copy */
 #define LNOCC_FAULT_ZERO_DIIS 2 /* fault injection: run without DIIS extrapolation */
+#define LNOCC_FAULT_NO_PLANES 4 /* fault injection: the (optional) allocations of FP64 digit planes fail */
 
 typedef struct lnocc_frag lnocc_frag; /* opaque: integrals, amplitudes and workspace of one fragment */
 

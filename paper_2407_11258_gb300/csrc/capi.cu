@@ -270,9 +270,13 @@ int lnocc_debug_gemm(int precision, int M, int N, int K, const double* A, const 
   if (!bf) {  // digit planes of an FP64 product
     const size_t nsl = lnocc::slice_ws_bytes(static_cast<size_t>(std::max(M, N)) * Kp * 8);
     lnocc::count_alloc();
-    LN_CUDA(cudaMalloc(&sl, nsl));
-    lnocc::split_ws().sl = sl;
-    lnocc::split_ws().sl_bytes = nsl;
+    if (cudaMalloc(&sl, nsl) == cudaSuccess) {
+      lnocc::split_ws().sl = sl;
+      lnocc::split_ws().sl_bytes = nsl;
+    } else {  // optional: the product runs on the SIMT kernel
+      cudaGetLastError();
+      sl = nullptr;
+    }
   }
   const lnocc::Ax one{1, 0};
   lnocc::pack(lnocc::view(A, one, one, lnocc::Ax{M, K}, one, one, lnocc::Ax{K, 1}), PA, s);

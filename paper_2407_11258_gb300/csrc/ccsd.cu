@@ -50,6 +50,15 @@ void Frag::dev_free(void* p) {
 void* Frag::alloc(size_t bytes, bool zero) {
   if (bytes == 0) bytes = 256;
   void* p = dev_alloc(bytes);
+  if (!p && slicews && !gexec) {  // the digit planes' workspace is optional: give it up first
+    dev_free(slicews);
+    allocs.erase(std::find(allocs.begin(), allocs.end(), slicews));
+    device_bytes -= static_cast<long long>(slicews_bytes);
+    slicews = nullptr;
+    slicews_bytes = 0;
+    use_workspace();
+    p = dev_alloc(bytes);
+  }
   if (!p) {
     oom = true;
     return nullptr;
@@ -257,8 +266,13 @@ int Frag::build(const double* eps_in, const double* B_in) {
   scrB = alloc(scr_bytes);
   splitk_cap = 1ull << 22;
   splitk = static_cast<double*>(alloc(splitk_cap * 8));
-  slicews_bytes = slice_ws_bytes(scr_bytes);
-  slicews = alloc(slicews_bytes);
+  // the digit planes of FP64 products are optional: without room for them those run on the SIMT kernel
+  if (!oom) {
+    const size_t n = slice_ws_bytes(scr_bytes);
+    slicews = opts.fault_inject & LNOCC_FAULT_NO_PLANES ? nullptr : alloc(n);
+    slicews_bytes = slicews ? n : 0;
+    oom = false;
+  }
   use_workspace();
   if (oom) {
     set_error("device allocation failed in lnocc_build_ints");

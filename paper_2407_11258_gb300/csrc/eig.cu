@@ -312,7 +312,7 @@ int sym_eig(double* A, double* V, double* w, int* order, int n, bool desc, doubl
   double hn[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if (n > 1) {
     // about one 2 x 2 block or row pair a thread, in one block per SM or, for larger orders, three (768 threads of
-    // 32 registers: all resident): order 333 26.4 and 26.6 ms with one and three, 500 61 and 54, 1000 299 and
+    // at most 40 registers: all resident): order 333 26.4 and 26.6 ms with one and three, 500 61 and 54, 1000 299 and
     // 222 (256 with eight: the barrier). A grid of tiles close to square keeps the angles each block needs few.
     const long long work = 1LL * h * h + 1LL * n * h;
     const int cap = num_sms() * (n > 400 ? 3 : 1);

@@ -45,11 +45,15 @@ struct Arena {
   std::vector<void*> ptrs;
   bool failed = false;
   void* get(size_t bytes) {
+    void* p = get_optional(bytes);
+    failed = failed || !p;
+    return p;
+  }
+  void* get_optional(size_t bytes) {
     void* p = nullptr;
     count_alloc();
     if (cudaMalloc(&p, std::max<size_t>(bytes, 256)) != cudaSuccess) {
       cudaGetLastError();
-      failed = true;
       return nullptr;
     }
     ptrs.push_back(p);
@@ -308,7 +312,7 @@ int finish(cudaStream_t s, int* dstatus, const char* who) {
   return LNOCC_OK;
 }
 
-struct SplitScope {  // split-K partials and FP64 digit planes, for the call's duration
+struct SplitScope {  // split-K partials and (where they fit) FP64 digit planes, for the call's duration
   SplitWs saved;
   // operand_bytes: the largest FP64-packed operand of the call (0: no FP64 products)
   SplitScope(Arena& ar, size_t operand_bytes) : saved(split_ws()) {
@@ -316,7 +320,7 @@ struct SplitScope {  // split-K partials and FP64 digit planes, for the call's d
     split_ws() = ws ? SplitWs{ws, size_t(1) << 22} : SplitWs{};
     if (operand_bytes > 0) {
       const size_t n = slice_ws_bytes(operand_bytes);
-      split_ws().sl = ar.get(n);
+      split_ws().sl = ar.get_optional(n);
       split_ws().sl_bytes = split_ws().sl ? n : 0;
     }
   }

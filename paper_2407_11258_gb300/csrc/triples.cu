@@ -768,7 +768,7 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     Packed* ops[4] = {&XT1, &XT2, &TO, &TOT};
     void* mem[4];
     const size_t n_mine = mine.size();
-    bool room = true;
+    bool room = !(opts.fault_inject & LNOCC_FAULT_NO_PLANES);
     for (int k = 0; k < 4 && room; ++k) {
       mem[k] = tmp_alloc(k < 2 ? tp.slxt : tp.slto);
       room = mem[k] != nullptr;
