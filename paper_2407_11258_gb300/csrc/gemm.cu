@@ -849,13 +849,14 @@ __device__ __forceinline__ void grp_epilogue(const TcArgs& p, const TileInfo& ti
         if (term == 0) {
           tma_store_5d(tW0, buf, 0, 2 * cc, 0, a0, ti.cz);
         } else {
-          if (term == 1 && cc == 0) bulk_wait_all();  // the region's stores are performed first
+          if (cc == 0) bulk_wait_all();  // the last term's copies are performed first
           if (term == 1)
             tma_reduce_add_5d(tW0, buf, 0, 2 * cc, 0, a0, ti.cz);
           else
             tma_reduce_add_5d(tW1, buf, 0, 0, 2 * cc, a0, ti.cz);
         }
       } else {
+        if (term == 1 && cc == 0) bulk_wait_all();
         tma_reduce_add_5d(tW0, buf, 0, 0, i0, a0, ti.cz + 2 * cc);
       }
       bulk_commit();
@@ -916,13 +917,14 @@ __device__ __forceinline__ void grp_epilogue32(const TcArgs& p, const TileInfo& 
         if (term == 0) {
           tma_store_5d(tW0, buf, 0, kk, 0, a0, ti.cz);
         } else {
-          if (term == 1 && ti.ct == 0 && cc == 0) bulk_wait_all();  // the region's stores are performed first
+          if (ti.ct == 0 && cc == 0) bulk_wait_all();  // the last term's copies are performed first
           if (term == 1)
             tma_reduce_add_5d(tW0, buf, 0, kk, 0, a0, ti.cz);
           else
             tma_reduce_add_5d(tW1, buf, 0, 0, kk, a0, ti.cz);
         }
       } else {
+        if (term == 1 && cc == 0) bulk_wait_all();
         tma_reduce_add_5d(tW0, buf, 0, 0, i0, a0, ti.cz + cc);
       }
       bulk_commit();

@@ -2,8 +2,9 @@
 //
 // One W chunk takes two launches. Kind 1 runs, per region (c, ta whole a values), sigma1 + sigma2 (two K
 // segments into one accumulator, stored), sigma3 and sigma5 (added); kind 2 runs, per region (ta whole (a, i)
-// pairs, a block of c), sigma4 and sigma6 (added). A region belongs to one CTA, so its additions follow its
-// store in one thread's order.
+// pairs, a block of c), sigma4 and sigma6 (added). A region belongs to one CTA, whose one copying thread waits
+// until the copies of a term are performed before it sends those of the next term: bulk copies of one thread are
+// not ordered by themselves, and FP32 additions in another order give other bits.
 //   * Rows: a 128-row tile holds ta = 128 / nocc whole a values (kind 1) or (a, i) pairs (kind 2) and starts at
 //     a multiple of ta nocc rows; the rows left over (at most nocc - 1) are computed and dropped.
 //   * Columns: whole values of the column's outer index (k, i or c), as many as fit 256 and evenly spread over
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(256, 1)
       }
       tc_fence_after();
       const uint32_t acc = tmem + buf * 256 + (static_cast<uint32_t>(ew * 32) << 16);
-      if (lead && g.kind == 1 && t.term == 1 && t.out0 == 0) bulk_wait_all();  // the region's stores come first
+      if (lead && t.term > 0 && t.out0 == 0) bulk_wait_all();  // the last term's copies are performed first
 #pragma unroll 1
       for (int x = 0; x < t.nout; ++x, nbox = nbox + 1 == p.nbox ? 0 : nbox + 1) {
         float v[32];
