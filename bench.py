@@ -69,7 +69,8 @@ def read_peaks():
 
 
 TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "k_gemm_tc_triples_traffic_nocc16_nvir240.md")
-TRAFFIC_SOURCES = ("paper_2407_11258_gb300/csrc/gemm.cu", "paper_2407_11258_gb300/csrc/triples.cu")
+TRAFFIC_SOURCES = ("paper_2407_11258_gb300/csrc/gemm.cu", "paper_2407_11258_gb300/csrc/triples.cu",
+                   "paper_2407_11258_gb300/csrc/triples_gemm.cu")
 
 
 def sources_digest():

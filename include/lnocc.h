@@ -51,7 +51,8 @@ extern "C" {
 #define LNOCC_PREC_MIXED 1 /* contractions as BF16x3 products with FP32 accumulation (tcgen05) */
 
 #define LNOCC_GUESS_MP2 0   /* t1 = 0, t2 = first-order amplitudes (Eq. 21, canonical form) */
-#define LNOCC_GUESS_GIVEN 1 /* start from t1_in / t2_in (restart / checkpoint resume) */
+#define LNOCC_GUESS_GIVEN 1 /* start from t1_in / t2_in (restart / checkpoint resume); t_ij^ab = t_ji^ba (an update
+                               takes the mean of the two) */
 #define LNOCC_GUESS_MLP 2   /* t1 = 0, t2 = learned guess of the model attached by lnocc_frag_set_mlp */
 
 /* (T) contraction launches on the mixed path. PER_TERM: one launch per W term (sigma1 + sigma2, sigma3,

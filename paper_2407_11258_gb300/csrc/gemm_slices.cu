@@ -16,12 +16,12 @@
 // than by the chain, a tenth plane holds |x| 2^-E, a tenth accumulator sums T, and an element with
 // T < 2^-9 sqrt(K) 2^(Ea+Eb), where the digits would give less, is summed in FP64 from the packed operands.
 // (At that line the digits' error is 0.5 2^-53 T.) T = 0 means that no nonzero meets another: zero exactly.
-// On the library's operands 0 to 0.3% of the elements fall below the line, in two products about half of them
-// (the (k,b) amplitude part of the dressed three-index terms, and the rotation of B into an active space,
-// whose rows decay away from their centre). With eight planes and no such check (128 x 64 tiles) 3 CCSD iterations
-// at (12, 96, 320) took 11.7 instead of 13.8 ms, (T) at (8, 64, 256) 15.1 instead of 18.2 ms (its 64-column products
-// take two tiles now) and the LNO space of (16, 160, 640) 13.9 instead of 21.3 ms (7.3 ms in the two products
-// that fall back), but an element 1e-16 of its row's largest was kept to 6e-3. The SIMT kernel: 131.6, 67.1, 30.4 ms.
+// On the library's operands 0 to 0.3% of the elements fall below the line; in three products, whose rows decay away
+// from a centre (amplitudes times F_vv, the two rotations of B into an active space), about half did, and those
+// run in K panels of 64 columns with exponents of their own (NarrowPanels). With eight planes and no such
+// check (128 x 64 tiles) 3 CCSD iterations at (12, 96, 320) took 11.7 instead of 13.5 ms, (T) at (8, 64, 256) 15.1
+// instead of 18.2 ms (its 64-column products take two tiles now) and the LNO space of (16, 160, 640) 14.0 instead
+// of 18.7 ms, but an element 1e-16 of its row's largest was kept to 6e-3. The SIMT kernel: 131.6, 67.1, 30.4 ms.
 // Rows whose chunk holds an infinity, a NaN, or only subnormal values are marked and summed in FP64 too.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -598,7 +598,7 @@ static void gemm_sliced_rows(const Sliced& A, int a_row0, const Sliced& B, int b
   constexpr int kcb = kChunk / kBK;
   if (!batch && !sym && nkb > 5) {
     // Split K over work items while they do not fill the SMs, the FP64 partials summed by the fixed-order
-    // reduction. A block of 32 columns is 1.8 us of MMAs; up to five of them cost less in one item than the
+    // reduction. A block of 32 columns is about 1.2 us of MMAs; up to five of them cost less in one item than the
     // reduction's launch (about 5 us) and half the MMAs.
     const SplitWs& w = split_ws();
     int kper = kcb;
@@ -651,13 +651,13 @@ bool gemm_f64_slices(const double* A, const double* B, int M, int N, int K, int 
   if (!w.sl || !dstatus) return false;
   unsigned char* base = static_cast<unsigned char*>(w.sl);
   const bool same = A == B && M == N;
-  if (same && slice_bytes(M, Kp) <= w.sl_bytes) {
+  if (same && slice_bytes(M, Kp) <= w.sl_bytes && (w.kw == 0 || Kp <= w.kw)) {
     const Sliced SA = slice_at(base, M, Kp, A, Kp);
     slice(SA, s);
     gemm_sliced_rows(SA, 0, SA, 0, M, N, K, C, 0, 0, nullptr, 1, 0, sym ? 1 : 0, 0, 0, s, dstatus);
     return true;
   }
-  const SlicePanels pl = plan_slice_panels(M, N, Kp, w.sl_bytes);
+  const SlicePanels pl = plan_slice_panels(M, N, Kp, w.sl_bytes, w.kw);
   if (pl.kw == 0) return false;
   OutMap Ck = C;
   for_each_slice_panel(pl, M, N, Kp, sym, [&](int k0, int kw, int n0, int nn, int m0, int mm, bool first) {

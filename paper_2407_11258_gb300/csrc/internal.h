@@ -149,8 +149,16 @@ struct SplitWs {
   size_t cap = 0;
   void* sl = nullptr;
   size_t sl_bytes = 0;
+  int kw = 0;  // FP64 products in K panels of at most so many columns (a multiple of 64; 0: any), see NarrowPanels
 };
 SplitWs& split_ws();
+// For FP64 products of operands whose rows decay away from a centre of their own: K panels of 64 columns. Every
+// panel of a row has its own exponent, so far fewer elements lie so far below the product of the rows'
+// largest that they have to be summed in FP64 (gemm_slices.cu).
+struct NarrowPanels {
+  NarrowPanels() { split_ws().kw = 64; }
+  ~NarrowPanels() { split_ws().kw = 0; }
+};
 // Bytes of a slice workspace for products whose operands take at most `operand_bytes` packed in FP64: room
 // for the planes of both (20 bytes an element) up to 256 MB (panels beyond that).
 inline size_t slice_ws_bytes(size_t operand_bytes) {

@@ -25,10 +25,11 @@ struct SlicePanels {
 // Invariant: slice_bytes(nb, kw) + slice_bytes(mb, kw) <= room. The K panel is the whole of K unless even a few
 // row tiles of it would not fit. B stays whole while it leaves a quarter of the workspace, and at least one row
 // tile of A, to the other operand; otherwise it is cut into panels of about half of the workspace. Whole tiles:
-// 128 rows of A, 64 of B.
-inline SlicePanels plan_slice_panels(int M, int N, int Kp, size_t room) {
+// 128 rows of A, 64 of B. kmax (a multiple of 64, or 0): the widest K panel the caller wants.
+inline SlicePanels plan_slice_panels(int M, int N, int Kp, size_t room, int kmax = 0) {
   SlicePanels p;
   if (M < 1 || N < 1 || Kp < 1) return p;
+  if (kmax > 0) Kp = std::min(Kp, kmax);
   auto fits = [&](int m, int n, int k) { return slice_bytes(m, k) + slice_bytes(n, k) <= room; };
   const int m1 = std::min(M, 512), n1 = std::min(N, 256);
   if (!fits(m1, n1, std::min(Kp, 2 * kSliceChunk))) return p;

@@ -41,6 +41,15 @@ extern "C" int check(int M, int N, int Kp, unsigned long long room, int sym) {
   }
   return bad;
 }
+extern "C" int narrow(int M, int N, int Kp, unsigned long long room, int kmax) {
+  const SlicePanels p = plan_slice_panels(M, N, Kp, room, kmax);
+  if (p.kw == 0) return -1;
+  int bad = p.kw > kmax;
+  for_each_slice_panel(p, M, N, Kp, false, [&](int k0, int kw, int n0, int nn, int m0, int mm, bool) {
+    if (slice_bytes(nn, kw) + slice_bytes(mm, kw) > room || kw > kmax || k0 + kw > Kp || n0 + nn > N || m0 + mm > M) bad = 1;
+  });
+  return bad;
+}
 extern "C" int sweep(const int* Ms, int nm, const int* Ns, int nn, const int* Ks, int nk, unsigned long long room, int sym,
                      int* at) {
   int plans = 0;
@@ -107,3 +116,9 @@ def test_panels_cover_small_products_once(planner):
 def test_workspace_that_cannot_hold_two_panels_is_refused(planner):
     for M, N, K in [(512, 256, 1024), (4000, 4000, 8192)]:
         assert planner.check(M, N, K, ctypes.c_ulonglong(1 << 20), 0) == -1
+
+
+def test_narrow_k_panels(planner):
+    for M, N, K in [(112640, 116, 192), (116, 74240, 192), (13824, 96, 128), (20, 30, 64), (5, 7, 1024)]:
+        for room in (2 << 20, 32 << 20, CAP):
+            assert planner.narrow(M, N, K, ctypes.c_ulonglong(room), 64) == 0
