@@ -48,6 +48,7 @@ extern "C" {
 #define LNOCC_PREC_FP64 0  /* every contraction in FP64 (plain GPU path): exact BF16 digit products on the tensor pipe,
                               rounded once; elements whose terms are all far below the product of their rows' largest
                               elements are summed in FP64, so that none is less exact than by an FP64 FMA chain */
+#define LNOCC_DEBUG_FAR 2  /* lnocc_debug_gemm only */
 #define LNOCC_PREC_MIXED 1 /* contractions as BF16x3 products with FP32 accumulation (tcgen05) */
 
 #define LNOCC_GUESS_MP2 0   /* t1 = 0, t2 = first-order amplitudes (Eq. 21, canonical form) */
@@ -232,7 +233,8 @@ int lnocc_frag_set_workspace(lnocc_frag* f, void* workspace, long long workspace
 
 /*
  * lnocc_debug_gemm -- diagnostic: C[M][N] = A[M][K] B[N][K]^T through the library's contraction engine
- * (operand packing + FP64 digit-plane GEMM, or BF16x3 tcgen05 GEMM with FP32 accumulation). Device pointers,
+ * (operand packing + FP64 digit-plane GEMM, or BF16x3 tcgen05 GEMM with FP32 accumulation; precision
+ * LNOCC_DEBUG_FAR: the FP64 GEMM with the twelve digits that products of far-apart rows take). Device pointers,
  * row-major FP64. Allocates its own temporaries and synchronizes `stream`. Not part of the method; it
  * lets the contraction kernels be checked on their own.
  */

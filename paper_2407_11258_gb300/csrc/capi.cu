@@ -281,6 +281,7 @@ int lnocc_debug_gemm(int precision, int M, int N, int K, const double* A, const 
   const lnocc::Ax one{1, 0};
   lnocc::pack(lnocc::view(A, one, one, lnocc::Ax{M, K}, one, one, lnocc::Ax{K, 1}), PA, s);
   lnocc::pack(lnocc::view(B, one, one, lnocc::Ax{N, K}, one, one, lnocc::Ax{K, 1}), PB, s);
+  lnocc::split_ws().far = precision == LNOCC_DEBUG_FAR ? lnocc::FarRows::kAll : lnocc::FarRows::kNone;
   lnocc::gemm(PA, PB, M, N, K, lnocc::out_rowmajor(C, N), s, dstatus);
   int st = 0;
   cudaError_t e = cudaMemcpyAsync(&st, dstatus, 4, cudaMemcpyDeviceToHost, s);

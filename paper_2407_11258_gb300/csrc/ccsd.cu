@@ -23,6 +23,7 @@
 
 #include "ccsd_kernels.h"
 #include "fragment.h"
+#include "gemm_slices.h"
 #include "internal.h"
 
 namespace lnocc {
@@ -541,15 +542,21 @@ void Frag::iterate(bool fp64_residual) {
   mark("g_aibj");
   // particle-particle ladder with the packed undressed integrals
   launch_ladder_ops(t2, C().Bp_t, C().Bm_t, o, v, s);
-  gemm(C().Vp, C().Bp_t, np_v, np_o, np_v, out_rowmajor(Lp_out, np_o), s, dstatus);
-  if (nm_v > 0 && nm_o > 0)
-    gemm(C().Vm, C().Bm_t, nm_v, nm_o, nm_v, out_rowmajor(Lm_out, nm_o), s, dstatus);
-  else cudaMemsetAsync(Lm_out, 0, 8, s);
+  {
+    const FarRows far_rows(v > kFarLadder ? FarRows::kAll : FarRows::kNone);
+    gemm(C().Vp, C().Bp_t, np_v, np_o, np_v, out_rowmajor(Lp_out, np_o), s, dstatus);
+    if (nm_v > 0 && nm_o > 0)
+      gemm(C().Vm, C().Bm_t, nm_v, nm_o, nm_v, out_rowmajor(Lm_out, nm_o), s, dstatus);
+    else cudaMemsetAsync(Lm_out, 0, 8, s);
+  }
   launch_ladder_unpack(Lp_out, Lm_out, Rsym, o, v, np_o, std::max(nm_o, 1), s);
   mark("ladder");
   // Wy[i][j][k][l] = Y_ij^kl = sum_cd (kc|ld) t_ij^cd ; Wb = g^_kilj + Y_ij^kl
-  contract_packed_b(view(t2, kOne, kOne, A(static_cast<int>(oo), vv), kOne, kOne, A(static_cast<int>(vv), 1)),
-                    C().kl_cd, static_cast<int>(oo), out_rowmajor(Wy, oo));
+  {
+    const FarRows far_rows(FarRows::kSmall);
+    contract_packed_b(view(t2, kOne, kOne, A(static_cast<int>(oo), vv), kOne, kOne, A(static_cast<int>(vv), 1)),
+                      C().kl_cd, static_cast<int>(oo), out_rowmajor(Wy, oo));
+  }
   gemm(K.PBoo, K.PBoo, static_cast<int>(oo), static_cast<int>(oo), N, OutMap{Wb, o, oo * o, 1, oo, o, o, 1.0, 0.0}, s,
        dstatus);
   permute(view(Wy, kOne, kOne, A(static_cast<int>(oo), oo), kOne, kOne, A(static_cast<int>(oo), 1)), Wb, 1.0, s);
@@ -565,19 +572,25 @@ void Frag::iterate(bool fp64_residual) {
   mark("hh_ladder");
   // ---- S (pre-P part)
   // Z_ij^kb = sum_cd (kc|bd) t_ij^cd ; S[i][j][a][b] = -sum_k t_k^a Z_ij^kb
-  contract_packed_b(view(t2, kOne, kOne, A(static_cast<int>(oo), vv), kOne, kOne, A(static_cast<int>(vv), 1)),
-                    C().kb_cd, static_cast<int>(ov), out_rowmajor(Z, ov));
+  {
+    const FarRows far_rows(v > kFarLadder ? FarRows::kAll : FarRows::kNone);
+    contract_packed_b(view(t2, kOne, kOne, A(static_cast<int>(oo), vv), kOne, kOne, A(static_cast<int>(vv), 1)),
+                      C().kb_cd, static_cast<int>(ov), out_rowmajor(Z, ov));
+  }
   mark("Z");
   contract(view(Z, kOne, A(static_cast<int>(oo), ov), A(v, 1), kOne, kOne, A(o, v)),
            view(t1, kOne, kOne, A(v, 1), kOne, kOne, A(o, v)), OutMap{S, vv, 1, 0, v, v, 1 << 30, -1.0, 0.0});
   mark("ZT");
   // E2: Fvv'_bc = F^_bc - sum_kld u_kl^bd (ld|kc); S += sum_c t_ij^ac Fvv'_bc
   permute(view(Fh + o * n + o, kOne, kOne, A(v, n), kOne, kOne, A(v, 1)), Fvv2, 0.0, s);
-  contract_packed_b(view(u, kOne, kOne, A(v, v), kOne, A(static_cast<int>(oo), vv), A(v, 1)), C().c_kld, v,
-                    out_rowmajor(Fvv2, v, -1.0, 1.0));
+  {
+    const FarRows far_rows(FarRows::kSmall);
+    contract_packed_b(view(u, kOne, kOne, A(v, v), kOne, A(static_cast<int>(oo), vv), A(v, 1)), C().c_kld, v,
+                      out_rowmajor(Fvv2, v, -1.0, 1.0));
+  }
   mark("Fvv");
   {
-    const NarrowPanels narrow;  // F is diagonally dominant: 3 iterations (12, 96, 320) 13.8 -> 13.5 ms
+    const FarRows far_rows(FarRows::kAll);  // F is diagonally dominant
     contract(view(t2, kOne, kOne, A(static_cast<int>(oo * v), v), kOne, kOne, A(v, 1)),
              view(Fvv2, kOne, kOne, A(v, v), kOne, kOne, A(v, 1)), out_rowmajor(S, v, 1.0, 1.0));
   }
@@ -588,9 +601,12 @@ void Frag::iterate(bool fp64_residual) {
   // sum_lcd u_lj^cd (kd|lc) = sum_{Q,d} B_Qkd Mtmp[Q][d][j]
   // (u rows taken as (i, d) with d contiguous so that the operand pack reads coalesced; the output
   // columns (i, d) land at Mtmp[Q][d][i])
-  contract(view(Bov, kOne, kOne, A(N, ov), kOne, kOne, A(static_cast<int>(ov), 1)),
-           view(u, kOne, A(o, vv), A(v, 1), kOne, A(o, o * vv), A(v, v)),
-           OutMap{Mtmp, 0, ov, 1, o, 1 << 30, v, 1.0, 0.0});
+  {
+    const FarRows far_rows(FarRows::kSmall);
+    contract(view(Bov, kOne, kOne, A(N, ov), kOne, kOne, A(static_cast<int>(ov), 1)),
+             view(u, kOne, A(o, vv), A(v, 1), kOne, A(o, o * vv), A(v, v)),
+             OutMap{Mtmp, 0, ov, 1, o, 1 << 30, v, 1.0, 0.0});
+  }
   contract(view(Bov, kOne, kOne, A(o, v), kOne, A(N, ov), A(v, 1)),
            view(Mtmp, kOne, kOne, A(o, 1), kOne, A(N, ov), A(v, o)), out_rowmajor(Foo2, o, 1.0, 1.0));
   mark("Foo");
@@ -603,25 +619,37 @@ void Frag::iterate(bool fp64_residual) {
   mark("E2b");
   // C2 intermediate X_kiac = g^_kiac - 1/2 sum_dl t_li^ad (kd|lc), stored [k][i][a][c]
   gemm(K.PBoo, K.PBvv, static_cast<int>(oo), static_cast<int>(vv), N, out_rowmajor(Xk, vv), s, dstatus);
-  contract_packed_b(view(t2, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)), C().kc_ld, static_cast<int>(ov),
-                    OutMap{Xk, vv, v, o * vv, 1, v, v, -0.5, 1.0});
+  {
+    const FarRows far_rows(FarRows::kSmall);
+    contract_packed_b(view(t2, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)), C().kc_ld, static_cast<int>(ov),
+                      OutMap{Xk, vv, v, o * vv, 1, v, v, -0.5, 1.0});
+  }
   mark("X");
   // Cp[(j,b),(i,a)] = sum_kc t_kj^bc X_kiac
-  contract(view(t2, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)),
-           view(Xk, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)), out_rowmajor(Cp, ov));
+  {
+    const FarRows far_rows(v > kFarRings ? FarRows::kAll : FarRows::kSmall);
+    contract(view(t2, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)),
+             view(Xk, kOne, A(o, vv), A(v, v), kOne, A(o, o * vv), A(v, 1)), out_rowmajor(Cp, ov));
+  }
   mark("Cp");
   // D2 intermediate Y[i][a][k][c] = 2 g^_aikc - g^_kiac + 1/2 sum_dl u_il^ad L_ldkc
   gemm(K.PBvo, K.PBov, static_cast<int>(ov), static_cast<int>(ov), N, OutMap{Yk, ov, ovv, 0, 1, o, 1 << 30, 2.0, 0.0},
        s, dstatus);
   gemm(K.PBoo, K.PBvv, static_cast<int>(oo), static_cast<int>(vv), N, OutMap{Yk, v, ovv, ov, 1, o, v, -1.0, 1.0}, s,
        dstatus);
-  contract_packed_b(view(u, kOne, A(o, o * vv), A(v, v), kOne, A(o, vv), A(v, 1)), C().L, static_cast<int>(ov),
-                    out_rowmajor(Yk, ov, 0.5, 1.0));
+  {
+    const FarRows far_rows(FarRows::kSmall);
+    contract_packed_b(view(u, kOne, A(o, o * vv), A(v, v), kOne, A(o, vv), A(v, 1)), C().L, static_cast<int>(ov),
+                      out_rowmajor(Yk, ov, 0.5, 1.0));
+  }
   mark("Yint");
   // S += 1/2 sum_kc u_jk^bc Y_aikc  -> rows (j,b), cols (i,a)
-  contract(view(u, kOne, A(o, o * vv), A(v, v), kOne, A(o, vv), A(v, 1)),
-           view(Yk, kOne, kOne, A(static_cast<int>(ov), ov), kOne, kOne, A(static_cast<int>(ov), 1)),
-           OutMap{S, vv, 1, o * vv, v, v, v, 0.5, 1.0});
+  {
+    const FarRows far_rows(v > kFarRings ? FarRows::kAll : FarRows::kSmall);
+    contract(view(u, kOne, A(o, o * vv), A(v, v), kOne, A(o, vv), A(v, 1)),
+             view(Yk, kOne, kOne, A(static_cast<int>(ov), ov), kOne, kOne, A(static_cast<int>(ov), 1)),
+             OutMap{S, vv, 1, o * vv, v, v, v, 0.5, 1.0});
+  }
 
   mark("D2");
   // ---- singles residual R1[i][a]

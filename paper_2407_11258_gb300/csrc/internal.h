@@ -149,15 +149,18 @@ struct SplitWs {
   size_t cap = 0;
   void* sl = nullptr;
   size_t sl_bytes = 0;
-  int kw = 0;  // FP64 products in K panels of at most so many columns (a multiple of 64; 0: any), see NarrowPanels
+  int far = 0;  // which FP64 products cut here take twelve digits instead of nine (FarRows)
 };
 SplitWs& split_ws();
-// For FP64 products of operands whose rows decay away from a centre of their own: K panels of 64 columns. Every
-// panel of a row has its own exponent, so far fewer elements lie so far below the product of the rows'
-// largest that they have to be summed in FP64 (gemm_slices.cu).
-struct NarrowPanels {
-  NarrowPanels() { split_ws().kw = 64; }
-  ~NarrowPanels() { split_ws().kw = 0; }
+// For FP64 products of operands whose rows decay away from centres of their own. With nine digits many elements lie
+// so far below the product of their rows' largest that they have to be summed in FP64 (gemm_slices.cu), with twelve
+// digits, at about twice the time of a product, hardly any. kSmall: only products so small that K is split below
+// a chunk of columns take them (each part has to stand for itself against the exponents of the whole chunk);
+// kAll: the rows can be far apart.
+struct FarRows {
+  enum { kNone, kSmall, kAll };
+  explicit FarRows(int which) { split_ws().far = which; }
+  ~FarRows() { split_ws().far = kNone; }
 };
 // Bytes of a slice workspace for products whose operands take at most `operand_bytes` packed in FP64: room
 // for the planes of both (20 bytes an element) up to 256 MB (panels beyond that).

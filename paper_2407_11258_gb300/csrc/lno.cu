@@ -420,6 +420,7 @@ extern "C" int lnocc_lno_densities(int precision, int kind, int nocc, int nvir, 
   LN_CUDA(cudaMemsetAsync(dstatus, 0, 16, s));
   const long long kpo = round_up(N, 64), kpd = static_cast<long long>(v) * round_up(static_cast<int>(std::min(ov, 1LL << 30)), 64);
   SplitScope split(ar, bf ? 0 : static_cast<size_t>(std::max(ov * kpo, kpd)) * 8);
+  const FarRows far(FarRows::kSmall);
   Engine eng{ar, bf, s, dstatus};
   count_launch(2);
   k_zero<<<grid1(1LL * o * o), 256, 0, s>>>(D_occ, 1LL * o * o);
@@ -617,9 +618,8 @@ extern "C" int lnocc_active_space(int precision, int nocc, int nvir, int naux, c
   k_rotate_cols<<<grid1(1LL * v * nv_F), 256, 0, s>>>(C_vir, v, nv_F, Rv, ov_, Cv, nv_F);
   k_block_diag<<<grid1(1LL * n * nF), 256, 0, s>>>(Co, o, no_F, Cv, v, nv_F, CF);
   SplitScope split(ar, precision == LNOCC_PREC_MIXED ? 0 : static_cast<size_t>(nq_h) * n * round_up(n, 64) * 8);
-  // the rows of B and the orbital coefficients are local in the orbital index, the coefficients graded as well: whole
-  // LNO space of (16, 160, 640) 21.4 -> 18.7 ms
-  const NarrowPanels narrow;
+  // the rows of B and the orbital coefficients are local in the orbital index, the coefficients graded as well
+  const FarRows far(FarRows::kAll);
   Engine eng{ar, precision == LNOCC_PREC_MIXED, s, dstatus};
   // per block of auxiliary indices Q (bounded packed operands):
   // H[Q][p][t] = sum_q B[Q][p][q] C_F[q][t]: rows (Q, p), K q; columns t (rows of C_F^T)

@@ -136,6 +136,23 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
   return d;
 }
 
+// The same for 32-byte rows (K blocks of 16 BF16) under the 32-byte swizzle: 8-row atoms 256 bytes apart.
+__device__ __forceinline__ uint64_t sdesc_sw32(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
+  d |= static_cast<uint64_t>(1) << 16;        // LBO = 16 B (ignored)
+  d |= static_cast<uint64_t>(256 >> 4) << 32; // SBO = 256 B
+  d |= static_cast<uint64_t>(1) << 46;        // descriptor version
+  d |= static_cast<uint64_t>(6) << 61;        // SWIZZLE_32B
+  return d;
+}
+// By the K block (BF16 columns of a row).
+template <int BK>
+__device__ __forceinline__ uint64_t sdesc_k(uint32_t saddr) {
+  static_assert(BK == 64 || BK == 32 || BK == 16, "row of 128, 64 or 32 bytes");
+  return BK == 64 ? sdesc_sw128(saddr) : BK == 32 ? sdesc_sw64(saddr) : sdesc_sw32(saddr);
+}
+
 // Instruction descriptor for kind::f16: BF16 x BF16 -> F32, both operands K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4)                                  // D format F32

@@ -476,7 +476,7 @@ __global__ void k_swap_outer_rows(const uint4* __restrict__ src, uint4* __restri
 //   * FP64: the digit planes of the four operands, cut once per call instead of in every product that reads them.
 //     An attached workspace without room for them, or a call whose allocations fail, runs without: sigma3, 4
 //     and 6 then cut their operands for every chunk into the handle's slice workspace, and the batched
-//     sigma1, 2 and 5 run on the SIMT kernel. The planes are left out beyond 32 GB (nocc 24 with nvir above 296).
+//     sigma1, 2 and 5 run on the SIMT kernel. The planes are left out beyond 32 GB (nocc 24 with nvir above 250).
 TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avail) {
   TriplesPlan p{};
   const long long oo = 1LL * o * o, vv = 1LL * v * v, ooo = oo * o;
@@ -527,7 +527,7 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avai
     }
   } else {
     const int Ktp = round_up(Kt, 64);
-    const size_t slxt = slice_bytes(vv * o, Ktp), slto = slice_bytes(v * oo, Ktp), planes = 2 * al(slxt) + 2 * al(slto);
+    const size_t slxt = slice_bytes(vv * o, Ktp, kFarDigits), slto = slice_bytes(v * oo, Ktp, kFarDigits), planes = 2 * al(slxt) + 2 * al(slto);
     p.total = p.need + (planes <= (size_t(32) << 30) ? planes : 0);
     p.alloc = p.total;
     if (p.total > p.need && (avail == 0 || avail >= p.total)) {
@@ -775,7 +775,8 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
     }
     if (room) {
       for (int k = 0; k < 4; ++k) {
-        sls[k] = slice_at(mem[k], ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp);
+        sls[k] = slice_at(mem[k], ops[k]->rows, ops[k]->Kp, static_cast<const double*>(ops[k]->p), ops[k]->Kp,
+                          kFarDigits);
         slice(sls[k], s);
         ops[k]->sl = &sls[k];
       }

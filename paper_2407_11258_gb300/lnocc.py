@@ -13,7 +13,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(PKG, "liblnocc.so")
 
 LNOCC_OK, LNOCC_EINVAL, LNOCC_ENOMEM, LNOCC_ENOCONV, LNOCC_ENUMERIC, LNOCC_ETIMEOUT, LNOCC_ECUDA = range(7)
-LNOCC_PREC_FP64, LNOCC_PREC_MIXED = 0, 1
+LNOCC_PREC_FP64, LNOCC_PREC_MIXED, LNOCC_DEBUG_FAR = 0, 1, 2
 LNOCC_GUESS_MP2, LNOCC_GUESS_GIVEN, LNOCC_GUESS_MLP = 0, 1, 2
 LNOCC_FAULT_NAN_INPUT, LNOCC_FAULT_ZERO_DIIS, LNOCC_FAULT_NO_PLANES = 1, 2, 4
 LNOCC_TK_AUTO, LNOCC_TK_PER_TERM, LNOCC_TK_GROUPED = 0, 1, 2

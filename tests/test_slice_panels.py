@@ -14,8 +14,8 @@ SRC = r"""
 using namespace lnocc;
 // -1: refused; 0: sound; 1: past the workspace; 2: a panel exceeds the operands or the plan; 3: an element of C and
 // a K panel not covered exactly once; 4: a B panel is read before it is cut
-extern "C" int check(int M, int N, int Kp, unsigned long long room, int sym) {
-  const SlicePanels p = plan_slice_panels(M, N, Kp, room);
+extern "C" int check(int M, int N, int Kp, unsigned long long room, int sym, int digits) {
+  const SlicePanels p = plan_slice_panels(M, N, Kp, room, digits);
   if (p.kw == 0) return -1;
   int bad = 0;
   long long area = 0, want = 0;
@@ -23,7 +23,7 @@ extern "C" int check(int M, int N, int Kp, unsigned long long room, int sym) {
   const int kpanels = (Kp + p.kw - 1) / p.kw;
   int cut_k = -1, cut_n = -1;
   for_each_slice_panel(p, M, N, Kp, sym != 0, [&](int k0, int kw, int n0, int nn, int m0, int mm, bool first) {
-    if (slice_bytes(nn, kw) + slice_bytes(mm, kw) > room) bad = bad ? bad : 1;
+    if (slice_bytes(nn, kw, digits) + slice_bytes(mm, kw, digits) > room) bad = bad ? bad : 1;
     if (kw < 1 || nn < 1 || mm < 1 || k0 + kw > Kp || n0 + nn > N || m0 + mm > M || nn > p.nb || mm > p.mb ||
         (k0 + kw < Kp && kw % kSliceChunk != 0) || k0 % kSliceChunk != 0)
       bad = bad ? bad : 2;
@@ -41,15 +41,6 @@ extern "C" int check(int M, int N, int Kp, unsigned long long room, int sym) {
   }
   return bad;
 }
-extern "C" int narrow(int M, int N, int Kp, unsigned long long room, int kmax) {
-  const SlicePanels p = plan_slice_panels(M, N, Kp, room, kmax);
-  if (p.kw == 0) return -1;
-  int bad = p.kw > kmax;
-  for_each_slice_panel(p, M, N, Kp, false, [&](int k0, int kw, int n0, int nn, int m0, int mm, bool) {
-    if (slice_bytes(nn, kw) + slice_bytes(mm, kw) > room || kw > kmax || k0 + kw > Kp || n0 + nn > N || m0 + mm > M) bad = 1;
-  });
-  return bad;
-}
 extern "C" int sweep(const int* Ms, int nm, const int* Ns, int nn, const int* Ks, int nk, unsigned long long room, int sym,
                      int* at) {
   int plans = 0;
@@ -57,9 +48,11 @@ extern "C" int sweep(const int* Ms, int nm, const int* Ns, int nn, const int* Ks
     for (int b = 0; b < nn; ++b)
       for (int c = 0; c < nk; ++c) {
         if (sym && Ms[a] != Ns[b]) continue;
-        const int r = check(Ms[a], Ns[b], Ks[c], room, sym);
-        if (r > 0) { at[0] = Ms[a], at[1] = Ns[b], at[2] = Ks[c], at[3] = r; return -1; }
-        plans += r == 0;
+        for (int digits : {kDigits, kFarDigits}) {
+          const int r = check(Ms[a], Ns[b], Ks[c], room, sym, digits);
+          if (r > 0) { at[0] = Ms[a], at[1] = Ns[b], at[2] = Ks[c], at[3] = r; return -1; }
+          plans += r == 0;
+        }
       }
   return plans;
 }
@@ -93,7 +86,7 @@ def test_panels_stay_inside_the_largest_workspace(planner):
     Ks = [k // 64 * 64 for k in (20000, 30000, 33700, 35000, 38000, 40000, 42048, 44000, 47040, 52000, 70016, 200000)]
     assert sweep(planner, Ms, Ns, Ks, CAP) > 0
     for M, N, K in [(100, 260, 47040), (130, 290, 42048), (144, 300, 40000), (92, 260, 95680), (120, 300, 162048)]:
-        assert planner.check(M, N, K, ctypes.c_ulonglong(CAP), 0) == 0
+        assert planner.check(M, N, K, ctypes.c_ulonglong(CAP), 0, 9) == 0
 
 
 def test_panels_stay_inside_any_workspace(planner):
@@ -115,10 +108,5 @@ def test_panels_cover_small_products_once(planner):
 
 def test_workspace_that_cannot_hold_two_panels_is_refused(planner):
     for M, N, K in [(512, 256, 1024), (4000, 4000, 8192)]:
-        assert planner.check(M, N, K, ctypes.c_ulonglong(1 << 20), 0) == -1
+        assert planner.check(M, N, K, ctypes.c_ulonglong(1 << 20), 0, 9) == -1
 
-
-def test_narrow_k_panels(planner):
-    for M, N, K in [(112640, 116, 192), (116, 74240, 192), (13824, 96, 128), (20, 30, 64), (5, 7, 1024)]:
-        for room in (2 << 20, 32 << 20, CAP):
-            assert planner.narrow(M, N, K, ctypes.c_ulonglong(room), 64) == 0
