@@ -154,7 +154,7 @@ struct SplitWs {
 SplitWs& split_ws();
 // For FP64 products of operands whose rows decay away from centres of their own. With nine digits many elements lie
 // so far below the product of their rows' largest that they have to be summed in FP64 (gemm_slices.cu), with twelve
-// digits, at about twice the time of a product, hardly any. kSmall: only products so small that K is split below
+// digits, at 1.2 to 2 times the time of a product (3840^3: 10.7 against 8.9 ms), hardly any. kSmall: only products so small that K is split below
 // a chunk of columns take them (each part has to stand for itself against the exponents of the whole chunk);
 // kAll: the rows can be far apart.
 struct FarRows {
