@@ -503,7 +503,8 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avai
   const long long cmb = chunk_mb > 0 ? chunk_mb : 768;
   auto set_rows = [&](int jp) {  // rows of W of jp elements
     p.jp = jp;
-    p.welems = std::max<long long>(std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab * oo * jp), v * oo * jp);
+    const long long most = std::min<long long>((cmb << 20) / static_cast<long long>(esz), max_slab * oo * jp);
+    p.welems = std::max<long long>(most, v * oo * jp);
     p.w = static_cast<size_t>(p.welems) * esz;
   };
   set_rows(o);
@@ -527,7 +528,8 @@ TriplesPlan triples_plan(int o, int v, int N, bool bf, int chunk_mb, size_t avai
     }
   } else {
     const int Ktp = round_up(Kt, 64);
-    const size_t slxt = slice_bytes(vv * o, Ktp, kFarDigits), slto = slice_bytes(v * oo, Ktp, kFarDigits), planes = 2 * al(slxt) + 2 * al(slto);
+    const size_t slxt = slice_bytes(vv * o, Ktp, kFarDigits), slto = slice_bytes(v * oo, Ktp, kFarDigits);
+    const size_t planes = 2 * al(slxt) + 2 * al(slto);
     p.total = p.need + (planes <= (size_t(32) << 30) ? planes : 0);
     p.alloc = p.total;
     if (p.total > p.need && (avail == 0 || avail >= p.total)) {
@@ -846,6 +848,8 @@ int Frag::triples(int nlo, const double* U, double* e_full, double* e_frag, doub
   const Packed* ops_a[4] = {&XT1, &TO, &XT2, &TOT};
   const Packed* ops_b[4] = {&TO, &XT2, &TO, &XT1};
   const int box_ab[4] = {128, 256, 128, 256};
+  // FP64 without planes: products that cut their operands per chunk take twelve digits like the planes
+  const FarRows far_rows(bf ? FarRows::kNone : FarRows::kAll);
   // tuning passes (t_max_chunks > 0) visit about t_max_chunks chunks spread over the plan
   const size_t chunk_stride = t_max_chunks > 0 ? std::max<size_t>(1, plan.size() / t_max_chunks) : 1;
   size_t chunk_idx = 0;
